@@ -7,25 +7,30 @@
 // Both query tiles consume every K/V tile, so each tile fetched from L2 feeds 256 rows.
 // Warp roles (384 threads = three warpgroups, one CTA per SM, 193 KB shared memory, all 512
 // TMEM columns; warpgroup 0 gives registers to the two softmax warpgroups with setmaxnreg):
-//   warp 0       TMA producers: lane 0 loads Q0/Q1 and the K tiles, lane 1 the V tiles, each
-//                into a two-stage ring (128 tokens x d, 128-byte swizzle, 64-element boxes);
+//   warp 0       TMA producer of Q0/Q1 and the K tiles, warp 2 of the V tiles, each into a
+//                two-stage ring (128 tokens x d, 128-byte swizzle, 64-element boxes);
 //                current-chunk tiles come from a 2-D map, history tiles from a 3-D map
 //                [block, token, channel] so a tile never reads past its block, or, with
 //                (1, 8, 8) spatial blocks of history frames, from a 4-D map
 //                [frame, y, x, channel] whose 8 x 8-token boxes put two routed blocks in one
 //                tile (rows 0-63 and 64-127; grid-edge tokens read as zero and are masked).
-//   warp 1       TMEM owner and single-thread UMMA issuer, order
-//                S0_0 S1_0 | PV0_0 S0_1 PV1_0 S1_1 | PV0_1 S0_2 PV1_1 S1_2 | ...
-//                (S_t = Q_t K^T, kind::f16, M=N=128, f32 in TMEM; PV_t: O_t += P_t V with P_t
-//                read from TMEM over the S_t columns and V read MN-major).
-//   warps 2, 3   idle (they complete warpgroup 0 for the register hand-over)
+//   warp 1       TMEM owner and UMMA issuer (S_t = Q_t K^T, kind::f16, M=N=128, f32 in TMEM;
+//                PV_t: O_t += P_t V with P_t read from TMEM and V read MN-major).
+//   warp 3       idle (it completes warpgroup 0 for the register hand-over)
 //   warps 4..7   softmax of Q0, warps 8..11 softmax of Q1: one query row per thread,
 //                tcgen05.ld of the S row, masking, exp2-domain online softmax with lazy
 //                rescaling (O_t and l rescaled only when the running max grows by more than
 //                8 = log2 256), P packed to bf16 and stored with tcgen05.st, epilogue O / l.
-// While one warpgroup runs its softmax the tensor core works on the other tile.  UMMAs of
-// one thread execute in issue order, so S_t for tile j+1 (issued after PV_t of tile j)
-// certifies that PV_t of tile j has completed: O_t may then be rescaled in place.
+// What bounds it: the tensor pipe (2,176 cycles per K/V tile for two query tiles, each UMMA 68)
+// against latency: ~300 cycles from the last UMMA of S until its softmax sees it, 200-400 for
+// the row's tcgen05.ld beside the other tile's PV, ~110 until the issuer acts on a barrier, and
+// ~1,600 for one softmax.  P has TMEM columns of its own, so an S buffer is free as soon as the
+// softmax has loaded its row, and S of the next query tile runs during this tile's softmax:
+//   S0 | S1 S0' PV0 S1' PV1 S0'' ...   (d = 128: both query tiles share one S buffer)
+// The chain per query tile is then S - load - S (1,265 cycles, 2,530 per K/V tile) instead of
+// softmax - PV - S (3,100 with P stored over S).  Measured on GB300 at the Matrix-Game-shaped
+// call (8 frames of 30x52, 12 heads of 128, 4 of 16 blocks): 537 -> 457 us, 1,570 TFLOP/s;
+// HY-World-shaped block step 12.4 -> 11.3 ms.  The arithmetic and its order are unchanged.
 // Load balance: a unit is one CTA's pair of query tiles with all its K/V tiles.  Units fill
 // whole rounds of one CTA per SM; the units of a last, partial round are split along the K/V
 // axis over all SMs, each part writes its unnormalised O with its row max and sum, and the
@@ -49,13 +54,13 @@ __device__ unsigned int g_attn_error;
 
 constexpr int BM = 128, BN = 128, kStages = 2;
 constexpr int kThreads = 384;
-// Registers: every thread starts with kLaunchRegs; warpgroup 0 (producer, MMA issuer, two
-// idle warps) drops to kRegsCtl and the softmax warpgroups rise to kRegsSoftmax.
+// Registers: every thread starts with kLaunchRegs; warpgroup 0 (producers, MMA issuer, one
+// idle warp) drops to kRegsCtl and the softmax warpgroups rise to kRegsSoftmax.
 constexpr int kLaunchRegs = 168, kRegsCtl = 96, kRegsSoftmax = 200;
 static_assert(128 * kRegsCtl + 256 * kRegsSoftmax <= kThreads * kLaunchRegs,
               "register split exceeds the launch allocation");
 static_assert(kThreads * kLaunchRegs <= 65536, "launch allocation exceeds the register file");
-constexpr int kTmemCols = 512;   // S0/P0 at 0, S1/P1 at 128, O0 at 256, O1 at 384
+constexpr int kTmemCols = 512;
 constexpr float kRescaleThreshold = 8.f;
 
 template <int HD>
@@ -67,6 +72,15 @@ struct Cfg {
   static constexpr int OFF_V = OFF_K + kStages * KV_BYTES;          // kStages V tiles
   static constexpr int OFF_BAR = OFF_V + kStages * KV_BYTES;
   static constexpr int SMEM = OFF_BAR + 256 + 1024;   // + barriers + alignment slack
+  // TMEM columns.  P has columns of its own (64 per query tile), so that an S buffer is free
+  // again once its softmax holds the row in registers.  d = 128: one S buffer (0), P at 128 and
+  // 192, O at 256 and 384.  d = 64: an S buffer per query tile (0, 128), P at 256 and 320, O at
+  // 384 and 448.
+  static constexpr int kSBufs = HD == 64 ? 2 : 1;
+  __host__ __device__ static constexpr uint32_t s_col(int t) { return kSBufs == 2 ? t * BN : 0; }
+  __host__ __device__ static constexpr uint32_t p_col(int t) { return kSBufs * BN + t * (BN / 2); }
+  __host__ __device__ static constexpr uint32_t o_col(int t) { return kSBufs * BN + BN + t * HD; }
+  static_assert((HD == 64 ? 2 : 1) * BN + BN + 2 * HD <= kTmemCols, "TMEM columns");
 };
 
 struct AttnKArgs {
@@ -76,7 +90,7 @@ struct AttnKArgs {
   int n_full;        // units run whole (CTAs 0 .. n_full-1)
   int n_split;       // parts of every remaining unit
   int chunk;         // K/V tiles per part
-  float* part_o;     // [tail unit][part][2][128][HD] unnormalised O of the parts
+  float* part_o;     // [tail unit][part][2][HD / 4][128][4] unnormalised O of the parts
   float* part_ml;    // [tail unit][part][2][128][2] row max (log2 domain) and row sum
   unsigned* counters;   // [tail unit] parts finished
   const int* idx;
@@ -92,7 +106,7 @@ struct AttnKArgs {
 struct Bars {
   uint64_t q_full;
   uint64_t k_full[kStages], k_empty[kStages], v_full[kStages], v_empty[kStages];
-  uint64_t s_full[2], p_full[2];
+  uint64_t s_full[2], s_free[2], p_full[2], pv_done[2];
   uint64_t fin, part_done, merge_go;
   uint32_t tmem_base;
   int abort;
@@ -251,7 +265,9 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     for (int t = 0; t < 2; ++t) {
       mbar_init(&bars->s_full[t], 1);
+      mbar_init(&bars->s_free[t], 128);
       mbar_init(&bars->p_full[t], 128);
+      mbar_init(&bars->pv_done[t], 1);
     }
     mbar_init(&bars->fin, 1);
     mbar_init(&bars->part_done, (has_q1 ? 2 : 1) * 128);
@@ -311,7 +327,9 @@ __global__ void __launch_bounds__(kThreads, 1)
           }
         }
       }
-    } else if (lane == 1) {
+    }
+  } else if (warp == 2) {
+    if (lane == 0) {
       tma_prefetch_desc(&tm_vc);
       tma_prefetch_desc(&tm_vh);
       bool waited = false;
@@ -344,73 +362,137 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ UMMA issuer
-    if (lane == 0) {
-      constexpr uint32_t idesc_qk = idesc_bf16_f32(BM, BN, false, false);
-      constexpr uint32_t idesc_pv = idesc_bf16_f32(BM, HD, false, true);
-      const uint32_t q_addr = smem_u32(sQ), k_addr = smem_u32(sK), v_addr = smem_u32(sV);
-      const int nq = has_q1 ? 2 : 1;
-      // Descriptors of the first k-slice of each operand; a k-slice, query tile or stage
-      // further on adds its byte offset / 16 to the 14-bit start-address field (the whole
-      // shared-memory window is below 256 KB, so the field never carries).  This keeps the
-      // single issuing thread at a few instructions per UMMA.
-      static_assert(C::SMEM + 1024 <= 256 * 1024, "descriptor start-address field would carry");
-      static_assert(BM == BN, "Q and K tiles share their k-slice offsets");
-      const uint64_t dq = sdesc_sw128(q_addr, 16, 1024);
-      const uint64_t dk = sdesc_sw128(k_addr, 16, 1024);
-      const uint64_t dv = sdesc_sw128(v_addr, BN * 128, 1024);
-      // S_t = Q_t K_j^T into the S_t columns (t * 128)
-      auto qk = [&](int t, int j) {
-        const uint64_t aq = dq + (uint64_t)((t * C::Q_BYTES) >> 4);
-        const uint64_t bk = dk + (uint64_t)(((j % kStages) * C::KV_BYTES) >> 4);
-#pragma unroll
-        for (int kk = 0; kk < HD / 16; ++kk) {
-          const uint64_t off = (uint64_t)(((kk >> 2) * (BM * 128) + (kk & 3) * 32) >> 4);
-          umma_bf16_ss(tmem + t * BN, aq + off, bk + off, idesc_qk, kk > 0 ? 1u : 0u);
-        }
-        umma_commit(&bars->s_full[t]);
+    // The warp stays converged (every lane waits, one elected lane issues) and every operand is
+    // warp-uniform, so that the UMMAs are issued from uniform registers: issued by one lane of a
+    // divergent branch they took ~50 cycles each, and S + PV of one tile 1,900 cycles.
+    constexpr uint32_t idesc_qk = idesc_bf16_f32(BM, BN, false, false);
+    constexpr uint32_t idesc_pv = idesc_bf16_f32(BM, HD, false, true);
+    const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);
+    const uint32_t sbase = __shfl_sync(0xffffffffu, smem_u32(smem), 0);
+    // Descriptors of the first k-slice of each operand; a k-slice, query tile or stage
+    // further on adds its byte offset / 16 to the 14-bit start-address field (the whole
+    // shared-memory window is below 256 KB, so the field never carries).
+    static_assert(C::SMEM + 1024 <= 256 * 1024, "descriptor start-address field would carry");
+    static_assert(BM == BN, "Q and K tiles share their k-slice offsets");
+    const uint64_t dq = sdesc_sw128(sbase + C::OFF_Q, 16, 1024);
+    const uint64_t dk = sdesc_sw128(sbase + C::OFF_K, 16, 1024);
+    const uint64_t dv = sdesc_sw128(sbase + C::OFF_V, BN * 128, 1024);
+    // Waits for the given phases of two barriers: half of the warp tests each, so that the
+    // usual case (both complete) costs one shared-memory round trip
+    auto wait2 = [&](uint64_t* b0, int ph0, uint64_t* b1, int ph1) -> bool {
+      uint64_t* const b = lane < 16 ? b0 : b1;
+      const uint32_t par = (uint32_t)(lane < 16 ? ph0 : ph1) & 1u;
+      if (__all_sync(0xffffffffu, mbar_try_wait(b, par))) return true;
+      const uint64_t t_begin = global_ns();
+      for (uint32_t it = 1;; ++it) {
+        if (__all_sync(0xffffffffu, mbar_try_wait(b, par))) return true;
+        if ((it & 63u) == 0u && __any_sync(0xffffffffu, aborted(bars) || global_ns() - t_begin > lim)) return false;
+      }
+    };
+    auto wait = [&](uint64_t* bar, int phase) -> bool { return wait2(bar, phase, bar, phase); };
+    const bool lead = elect_one();   // the same lane issues and commits everything
+    // S_t = Q_t K_j^T into the S columns of tile t.  The two barriers of the PV that follows are
+    // tested before the last three UMMAs: at ~165 cycles a wait, testing them after S left the
+    // tensor pipe idle for that long on every tile (Matrix-Game-shaped call 482 -> 464 us).
+    auto issue_s = [&](const int t, int j, uint64_t* b0, int ph0, uint64_t* b1, int ph1) -> bool {
+      tc_fence_after();
+      const uint64_t aq = dq + (uint64_t)((t * C::Q_BYTES) >> 4);
+      const uint64_t bk = dk + (uint64_t)((j % kStages) * (C::KV_BYTES >> 4));
+      auto umma = [&](int kk) {
+        const uint64_t off = (uint64_t)(((kk >> 2) * (BM * 128) + (kk & 3) * 32) >> 4);
+        umma_bf16_ss(tm + C::s_col(t), aq + off, bk + off, idesc_qk, kk > 0 ? 1u : 0u);
       };
-      // O_t += P_t V_j, P_t read from TMEM over the S_t columns
-      auto pv = [&](int t, int j) {
-        const uint64_t bv = dv + (uint64_t)(((j % kStages) * C::KV_BYTES) >> 4);
+      constexpr int nk = HD / 16;
+      if (lead) {
+#pragma unroll
+        for (int kk = 0; kk < nk - 3; ++kk) umma(kk);
+      }
+      __syncwarp();
+      const bool r = mbar_try_wait(lane < 16 ? b0 : b1, (uint32_t)(lane < 16 ? ph0 : ph1) & 1u);
+      if (lead) {
+#pragma unroll
+        for (int kk = nk - 3; kk < nk; ++kk) umma(kk);
+        umma_commit(&bars->s_full[t]);
+      }
+      __syncwarp();
+      return __all_sync(0xffffffffu, r);
+    };
+    // O_t += P_t V_j, P_t read from TMEM
+    auto issue_pv = [&](const int t, int j) {
+      tc_fence_after();
+      if (lead) {
+        const uint64_t bv = dv + (uint64_t)((j % kStages) * (C::KV_BYTES >> 4));
 #pragma unroll
         for (int kk = 0; kk < BN / 16; ++kk)
-          umma_bf16_ts(tmem + 256 + t * 128, tmem + t * BN + kk * 8,
-                       bv + (uint64_t)((kk * 16 * 128) >> 4), idesc_pv, (j > 0 || kk > 0) ? 1u : 0u);
-      };
-      bool ok = mbar_wait(&bars->q_full, 0, lim) && mbar_wait(&bars->k_full[0], 0, lim);
-      tc_fence_after();
-      if (ok && n_tiles > 0) {
-        for (int t = 0; t < nq; ++t) qk(t, 0);
-        umma_commit(&bars->k_empty[0]);
+          umma_bf16_ts(tm + C::o_col(t), tm + C::p_col(t) + kk * 8, bv + (uint64_t)((kk * 16 * 128) >> 4),
+                       idesc_pv, (j > 0 || kk > 0) ? 1u : 0u);
+        umma_commit(&bars->pv_done[t]);
       }
+      __syncwarp();
+    };
+    auto kf = [&](int j) { return &bars->k_full[j % kStages]; };
+    auto vf = [&](int j) { return &bars->v_full[j % kStages]; };
+    uint64_t *const sf0 = &bars->s_free[0], *const sf1 = &bars->s_free[1];
+    uint64_t *const pf0 = &bars->p_full[0], *const pf1 = &bars->p_full[1];
+    bool ok = n_tiles > 0 && wait2(&bars->q_full, 0, kf(0), 0);
+    if (ok) issue_s(0, 0, pf0, 0, pf0, 0);
+    if (!has_q1) {
+      // one query tile: S of tile j+1 runs during the softmax of tile j
       for (int j = 0; ok && j < n_tiles; ++j) {
-        const int s = j % kStages;
-        const uint32_t ph = (uint32_t)j & 1u;
-        const bool more = j + 1 < n_tiles;
-        // K_{j+1} is awaited with V_j, while P_0 is still being formed, so that S_0 of tile
-        // j+1 follows PV_0 of tile j without a wait (its load was released two tiles ago)
-        if (aborted(bars) || !mbar_wait(&bars->v_full[s], (uint32_t)(j / kStages) & 1u, lim) ||
-            (more && !mbar_wait(&bars->k_full[(j + 1) % kStages], (uint32_t)((j + 1) / kStages) & 1u, lim)) ||
-            !mbar_wait(&bars->p_full[0], ph, lim)) { ok = false; break; }
-        tc_fence_after();
-        pv(0, j);
-        if (more) qk(0, j + 1);
-        if (nq == 2) {
-          if (aborted(bars) || !mbar_wait(&bars->p_full[1], ph, lim)) { ok = false; break; }
-          tc_fence_after();
-          pv(1, j);
+        bool ready = false;
+        if (j + 1 < n_tiles) {
+          if (!(ok = wait2(kf(j + 1), (j + 1) / kStages, sf0, j))) break;
+          ready = issue_s(0, j + 1, vf(j), j / kStages, pf0, j);
         }
-        umma_commit(&bars->v_empty[s]);
-        if (more) {
-          if (nq == 2) qk(1, j + 1);
-          umma_commit(&bars->k_empty[(j + 1) % kStages]);
-        }
+        if (!ready && !(ok = wait2(vf(j), j / kStages, pf0, j))) break;
+        issue_pv(0, j);
       }
-      if (!ok) set_abort(bars);
-      // every issued UMMA has completed before the epilogue reads O and TMEM is released
-      umma_commit(&bars->fin);
-      mbar_wait(&bars->fin, 0, lim);
+    } else if (C::kSBufs == 2) {
+      // S0 S1 | S0' PV0 S1' PV1 | ...: a tile's next S waits for its own columns only
+      if (ok) issue_s(1, 0, pf0, 0, pf0, 0);
+      for (int j = 0; ok && j < n_tiles; ++j) {
+        const bool more = j + 1 < n_tiles;
+        bool ready = false;
+        if (more) {
+          if (!(ok = wait2(kf(j + 1), (j + 1) / kStages, sf0, j))) break;
+          ready = issue_s(0, j + 1, vf(j), j / kStages, pf0, j);
+        }
+        if (!ready && !(ok = wait2(vf(j), j / kStages, pf0, j))) break;
+        issue_pv(0, j);
+        ready = false;
+        if (more) {
+          if (!(ok = wait(sf1, j))) break;
+          ready = issue_s(1, j + 1, pf1, j, pf1, j);
+        }
+        if (!ready && !(ok = wait(pf1, j))) break;
+        issue_pv(1, j);
+      }
+    } else {
+      // S0 | S1 S0' PV0 S1' PV1 S0'' ...: the next S runs as soon as the softmax before it has
+      // read the shared S columns, ahead of the PV of the tile before that
+      for (int j = 0; ok && j < n_tiles; ++j) {
+        if (!(ok = wait(sf0, j))) break;
+        bool ready = issue_s(1, j, pf1, j - 1, pf1, j - 1);
+        if (j > 0) {
+          if (!ready && !(ok = wait(pf1, j - 1))) break;
+          issue_pv(1, j - 1);
+        }
+        ready = false;
+        if (j + 1 < n_tiles) {
+          if (!(ok = wait2(kf(j + 1), (j + 1) / kStages, sf1, j))) break;
+          ready = issue_s(0, j + 1, vf(j), j / kStages, pf0, j);
+        }
+        if (!ready && !(ok = wait2(vf(j), j / kStages, pf0, j))) break;
+        issue_pv(0, j);
+      }
+      if (ok && (ok = wait(pf1, n_tiles - 1))) issue_pv(1, n_tiles - 1);
     }
+    if (!ok && lane == 0) set_abort(bars);
+    // every issued UMMA has completed before the epilogue reads O and TMEM is released
+    if (lead) umma_commit(&bars->fin);
+    __syncwarp();
+    mbar_wait(&bars->fin, 0, lim);
+    __syncwarp();
   }
   // the last UMMA has completed (fin) and every softmax thread has read TMEM
   tc_fence_before();
@@ -424,29 +506,55 @@ __global__ void __launch_bounds__(kThreads, 1)
   if (warp < 8 || has_q1) {
     // ------------------------------------------------------------ softmax + epilogue
     const int t = warp < 8 ? 0 : 1;
+    const bool last_tile = t == (has_q1 ? 1 : 0);
     const int q4 = warp & 3;
     const int row = q4 * 32 + lane;
     const uint32_t tl = tmem + ((uint32_t)(q4 * 32) << 16);
-    const uint32_t colS = t * BN, colO = 256 + t * 128;
+    const uint32_t colS = C::s_col(t), colP = C::p_col(t), colO = C::o_col(t);
     float m_ref = -INFINITY, l = 0.f;
     bool ok = true;
     bool waited = false;
+    // A phase of one barrier for the whole warp: one test in the usual case
+    auto warp_wait = [&](uint64_t* bar, uint32_t parity) -> bool {
+      if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+      const uint64_t t_begin = global_ns();
+      for (uint32_t it = 1;; ++it) {
+        if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+        if ((it & 63u) == 0u && __any_sync(0xffffffffu, aborted(bars) || global_ns() - t_begin > lim)) return false;
+      }
+    };
+    // K/V tile of the current history block (counted, so that no division sits in the loop)
+    int blk_tile = k0 > a.n_cur_tiles && a.tiles_per_block > 0 ? (k0 - a.n_cur_tiles) % a.tiles_per_block : 0;
     for (int j = 0; j < n_tiles; ++j) {
       const int jg = k0 + j;   // global K/V tile
+      const bool hist = jg >= a.n_cur_tiles;
+      const uint32_t par = (uint32_t)j & 1u;
       // spatial history tile: the routed block indices are fetched before the wait
-      int sm0 = -1, sm1 = -1;
-      if (a.spatial && jg >= a.n_cur_tiles) {
+      int sm0 = -1, sm1 = -1, valid = BN;
+      if (!hist) {
+        valid = min(BN, a.cur_rows - jg * BN);
+      } else if (a.spatial) {
         wait_routing(waited);
         const int jj = jg - a.n_cur_tiles;
         sm0 = routed_block(a, i, h, 2 * jj);
         sm1 = 2 * jj + 1 < a.K_eff ? routed_block(a, i, h, 2 * jj + 1) : -1;
+      } else {
+        valid = min(BN, a.B_v - blk_tile * BN);
+        if (++blk_tile == a.tiles_per_block) blk_tile = 0;
       }
-      bool w = !aborted(bars) && mbar_wait(&bars->s_full[t], (uint32_t)j & 1u, lim);
-      if (!__all_sync(0xffffffffu, w)) { ok = false; break; }
+      if (!warp_wait(&bars->s_full[t], par)) { ok = false; break; }
       tc_fence_after();
+      // the last query tile's S has read the K stage: the softmax hands it back, which keeps
+      // that commit off the UMMA issuer (~70 cycles each)
       uint32_t sr[BN];
-      tmem_ld_x64(tl + colS, sr);
-      tmem_ld_x64(tl + colS + 64, sr + 64);
+      tmem_ld_x64_async(tl + colS, sr);
+      tmem_ld_x64_async(tl + colS + 64, sr + 64);
+      tmem_wait_ld_x64(sr);
+      tmem_wait_ld_x64(sr + 64);
+      // S is in registers: its columns go back to the issuer
+      tc_fence_before();
+      mbar_arrive(&bars->s_free[t]);
+      if (last_tile && q4 == 1 && lane == 0) mbar_arrive(&bars->k_empty[j % kStages]);
       if (sm0 >= 0) {
         // key positions outside a truncated block, and the unused half of a last odd tile
         const uint64_t v0 = spatial_block(a, sm0).valid;
@@ -457,20 +565,11 @@ __global__ void __launch_bounds__(kThreads, 1)
           for (int c = 0; c < BN; ++c)
             if (!((w4[c >> 5] >> (c & 31)) & 1u)) sr[c] = __float_as_uint(-INFINITY);
         }
-      } else {
-        int valid;
-        if (jg < a.n_cur_tiles) {
-          valid = min(BN, a.cur_rows - jg * BN);
-        } else {
-          const int jj = jg - a.n_cur_tiles;
-          valid = min(BN, a.B_v - (jj % a.tiles_per_block) * BN);
-        }
+      } else if (valid < BN) {
         // columns past the chunk / block end (only in a ragged last tile) get -inf
-        if (valid < BN) {
 #pragma unroll
-          for (int c = 0; c < BN; ++c)
-            if (c >= valid) sr[c] = __float_as_uint(-INFINITY);
-        }
+        for (int c = 0; c < BN; ++c)
+          if (c >= valid) sr[c] = __float_as_uint(-INFINITY);
       }
       // raw-logit max (scale > 0 commutes with max): 3-input max, 8 independent chains
       float m8[8];
@@ -491,26 +590,36 @@ __global__ void __launch_bounds__(kThreads, 1)
         l *= corr;
       }
       // P = 2^(s * scale_log2 - m_ref): packed f32x2 FMA and sums, one MUFU op per element,
-      // packed to bf16 pairs over the first 64 S columns of this lane
+      // packed to bf16 pairs and stored in two halves, the first while the second is formed.
+      // PV of the previous K/V tile must have read P_t (and completed O_t) before: tested here,
+      // where it normally has, and looked at after the first half.
+      bool pv_ok = j == 0 || mbar_try_wait(&bars->pv_done[t], par ^ 1u);
       const float2 sc2 = make_float2(a.scale_log2, a.scale_log2);
       const float2 nm2 = make_float2(-m_ref, -m_ref);
       float2 s4[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f),
                       make_float2(0.f, 0.f)};
 #pragma unroll
-      for (int c = 0; c < BN; c += 2) {
-        const float2 x = __ffma2_rn(make_float2(__uint_as_float(sr[c]), __uint_as_float(sr[c + 1])),
-                                    sc2, nm2);
-        const float2 p = make_float2(ex2_approx(x.x), ex2_approx(x.y));
-        s4[(c >> 1) & 3] = __fadd2_rn(s4[(c >> 1) & 3], p);
-        __nv_bfloat162 b2 = __floats2bfloat162_rn(p.x, p.y);
-        sr[c / 2] = *reinterpret_cast<uint32_t*>(&b2);
+      for (int half = 0; half < 2; ++half) {
+#pragma unroll
+        for (int c = half * 64; c < half * 64 + 64; c += 2) {
+          const float2 x = __ffma2_rn(make_float2(__uint_as_float(sr[c]), __uint_as_float(sr[c + 1])),
+                                      sc2, nm2);
+          const float2 p = make_float2(ex2_approx(x.x), ex2_approx(x.y));
+          s4[(c >> 1) & 3] = __fadd2_rn(s4[(c >> 1) & 3], p);
+          __nv_bfloat162 b2 = __floats2bfloat162_rn(p.x, p.y);
+          sr[c / 2] = *reinterpret_cast<uint32_t*>(&b2);
+        }
+        if (half == 0) {
+          if (!__all_sync(0xffffffffu, pv_ok)) pv_ok = warp_wait(&bars->pv_done[t], par ^ 1u);
+          tc_fence_after();
+        }
+        if (pv_ok) tmem_st_x32_async(tl + colP + half * 32, sr + half * 32);
       }
+      if (!pv_ok) { ok = false; break; }
+      if (j > 0 && last_tile && q4 == 0 && lane == 0) mbar_arrive(&bars->v_empty[(j - 1) % kStages]);
       const float2 s2 = __fadd2_rn(__fadd2_rn(s4[0], s4[1]), __fadd2_rn(s4[2], s4[3]));
       l += s2.x + s2.y;
-      tmem_st_x64(tl + colS, sr);
       if (j > 0 && __any_sync(0xffffffffu, need)) {
-        // O_t holds P_0..P_{j-1} V and is final: S_t of tile j was issued after PV_t of
-        // tile j-1, and PV_t of tile j waits for p_full below
 #pragma unroll
         for (int half = 0; half < HD / 64; ++half) {
           uint32_t orr[64];
@@ -520,6 +629,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           tmem_st_x64(tl + colO + half * 64, orr);
         }
       }
+      tmem_wait_st();
       tc_fence_before();
       mbar_arrive(&bars->p_full[t]);
     }
@@ -569,16 +679,22 @@ __global__ void __launch_bounds__(kThreads, 1)
     } else {
       // this part's unnormalised O with its row max (log2 domain) and row sum
       const int64_t slot0 = ((int64_t)tail_unit * a.n_split) * 2 * BM + t * BM + row;
+      // O of part p, columns 4 c .. 4 c + 3 of this row: column groups of 128 rows, so that a
+      // warp's 16-byte accesses are contiguous (row by row they touched 32 lines each, and
+      // merging three parts of 128 x 64 took 8 us)
+      auto part_o = [&](int p, int c) -> float4* {
+        const int64_t tile = ((int64_t)tail_unit * a.n_split + p) * 2 + t;
+        return reinterpret_cast<float4*>(a.part_o) + (tile * (HD / 4) + c) * BM + row;
+      };
       if (ok) {
         const int64_t slot = slot0 + (int64_t)part * 2 * BM;
 #pragma unroll
         for (int half = 0; half < HD / 64; ++half) {
           uint32_t orr[64];
           tmem_ld_x64(tl + colO + half * 64, orr);
-          float4* dst = reinterpret_cast<float4*>(a.part_o + slot * HD + half * 64);
 #pragma unroll
           for (int c = 0; c < 64; c += 4)
-            __stcg(dst + c / 4, make_float4(__uint_as_float(orr[c]), __uint_as_float(orr[c + 1]),
+            __stcg(part_o(part, half * 16 + c / 4), make_float4(__uint_as_float(orr[c]), __uint_as_float(orr[c + 1]),
                                             __uint_as_float(orr[c + 2]), __uint_as_float(orr[c + 3])));
         }
         __stcg(reinterpret_cast<float2*>(a.part_ml) + slot, make_float2(m_ref, l));
@@ -617,10 +733,9 @@ __global__ void __launch_bounds__(kThreads, 1)
           for (int p = 0; p < a.n_split; ++p) {
             const int64_t sp = slot0 + (int64_t)p * 2 * BM;
             const float wgt = ex2_approx(__ldcg(ml + sp).x - mm);
-            const float4* src = reinterpret_cast<const float4*>(a.part_o + sp * HD + half * 64);
 #pragma unroll
             for (int c = 0; c < 64; c += 4) {
-              const float4 v = __ldcg(src + c / 4);
+              const float4 v = __ldcg(part_o(p, half * 16 + c / 4));
               acc[c] = fmaf(wgt, v.x, acc[c]);
               acc[c + 1] = fmaf(wgt, v.y, acc[c + 1]);
               acc[c + 2] = fmaf(wgt, v.z, acc[c + 2]);
