@@ -608,6 +608,7 @@ cast_status cast_ffn_step(const cast_ffn_args* a, void* ws, size_t ws_bytes, voi
   g2.K = a->D_ff;
   g2.n_anchors = a->n_anchors;
   g2.gelu = false;
+  g2.after_gemm = true;
   for (int i = 0; i < a->n_anchors; ++i) {
     g1.a_frame[i] = a->anchors[i];
     g1.c_frame[i] = i;
