@@ -165,7 +165,7 @@ cast_status validate_route(const cast_route_args* a) {
   if (route_pool_smem_bytes(*a) > 200 * 1024)
     return fail(CAST_ERR_UNSUPPORTED, "%s: H*d = %d channels exceed the pooling kernel's shared memory",
                 who, a->H * a->d);
-  if (a->M > 0 && route_head_smem_bytes(*a) > 200 * 1024)
+  if (a->M > 0 && route_head_limit_bytes(*a) > 200 * 1024)
     return fail(CAST_ERR_UNSUPPORTED, "%s: %d anchors x %d blocks exceed the per-head shared memory",
                 who, a->n_anchors, a->M);
   return CAST_OK;

@@ -78,6 +78,8 @@ RoutePlan route_plan(const cast_route_args& a);
 // (pooled query, o_bar, pi, keys and masks of every anchor of one head)
 size_t route_pool_smem_bytes(const cast_route_args& a);
 size_t route_head_smem_bytes(const cast_route_args& a);
+// what the 200 KB limit of the per-head state counts
+size_t route_head_limit_bytes(const cast_route_args& a);
 // Arguments must have been validated; ws holds at least route_plan(a).total_bytes.
 cast_status launch_route(const cast_route_args& a, void* ws, cudaStream_t st);
 // Nonzero when a routing kernel met a candidate index outside [0, M) or repeated in its set.

@@ -397,8 +397,91 @@ __device__ __forceinline__ bool in_topk(const float* key, int M, int K, int m) {
 // Warp-wide sum of one value per lane (every lane gets the total).
 __device__ __forceinline__ float warp_total(float v) { return warp_sum(v); }
 
+// Omission scores with a Gram matrix, u = coef^2 e^T G e with e = o_bar_i - v_bar_m (Eq.
+// omission), of the pairs p = i * nm + ml (anchor i, block ml of this CTA).  Every thread of the
+// CTA calls it.  A warp takes kGramPairs pairs at once and lane l the rows l, l + 32, ... of G:
+// columns are staged kGramCols at a time (rows padded by one float: conflict-free), read by every
+// warp, and each value feeds all of a warp's pairs from registers, so that the FMAs bound it
+// (na * nm * d^2 of them).  Reading G from global memory row by row instead, each lane its own
+// row, cost 613 us for 12 heads of 4 anchors x 16 blocks (2,290 us for the projected
+// Matrix-Game-shaped block step).  y_r sums over c in order and the rows of a lane in order, as
+// before: the scores are the same bits.
+constexpr int kGramPairs = 8, kGramCols = 32;
+__host__ __device__ constexpr size_t gram_stage_bytes(int d) { return (size_t)d * (kGramCols + 1) * sizeof(float); }
+
+template <int HD>
+__device__ void gram_scores(const float* __restrict__ G, const float* ob, const float* v, int64_t v_stride,
+                            int na, int nm, int out_stride, const float* pi, float eps, float* gs, float* out) {
+  constexpr int R = HD / 32, kPer = HD * kGramCols / 4 / kHeadThreads;   // float4 loads per thread and stage
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int n_pairs = na * nm;
+  constexpr int kBatch = kHeadWarps * kGramPairs;
+  for (int b0 = 0; b0 < n_pairs; b0 += kBatch) {
+    const float *op[kGramPairs], *vp[kGramPairs];
+    float y[kGramPairs][R];
+#pragma unroll
+    for (int k = 0; k < kGramPairs; ++k) {
+      const int p = min(b0 + warp * kGramPairs + k, n_pairs - 1), i = p / nm;
+      op[k] = ob + i * HD;
+      vp[k] = v + (int64_t)(p - i * nm) * v_stride;
+#pragma unroll
+      for (int r = 0; r < R; ++r) y[k][r] = 0.f;
+    }
+    for (int c0 = 0; c0 < HD; c0 += kGramCols) {
+      float4 g4[kPer];
+#pragma unroll
+      for (int t = 0; t < kPer; ++t) {
+        const int e = tid + t * kHeadThreads;
+        g4[t] = __ldg(reinterpret_cast<const float4*>(G + (int64_t)(e >> 3) * HD + c0) + (e & 7));
+      }
+      __syncthreads();   // the stage before has been read
+#pragma unroll
+      for (int t = 0; t < kPer; ++t) {
+        const int e = tid + t * kHeadThreads;
+        float* d = gs + (e >> 3) * (kGramCols + 1) + (e & 7) * 4;
+        d[0] = g4[t].x; d[1] = g4[t].y; d[2] = g4[t].z; d[3] = g4[t].w;
+      }
+      __syncthreads();
+      if (b0 + warp * kGramPairs < n_pairs) {
+#pragma unroll 2
+        for (int c = 0; c < kGramCols; c += 4) {
+          float g[4][R];
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+#pragma unroll
+            for (int r = 0; r < R; ++r) g[q][r] = gs[(lane + 32 * r) * (kGramCols + 1) + c + q];
+#pragma unroll
+          for (int k = 0; k < kGramPairs; ++k) {
+            const float4 o4 = *reinterpret_cast<const float4*>(op[k] + c0 + c);
+            const float4 v4 = *reinterpret_cast<const float4*>(vp[k] + c0 + c);
+            const float e[4] = {o4.x - v4.x, o4.y - v4.y, o4.z - v4.z, o4.w - v4.w};
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+#pragma unroll
+              for (int r = 0; r < R; ++r) y[k][r] = fmaf(g[q][r], e[q], y[k][r]);
+          }
+        }
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < kGramPairs; ++k) {
+      const int p = b0 + warp * kGramPairs + k;
+      if (p >= n_pairs) break;   // uniform across the warp
+      float acc = 0.f;
+#pragma unroll
+      for (int r = 0; r < R; ++r) acc = fmaf(op[k][lane + 32 * r] - vp[k][lane + 32 * r], y[k][r], acc);
+      acc = warp_sum(acc);
+      if (lane == 0) {
+        const int i = p / nm, q = i * out_stride + (p - i * nm);
+        const float coef = pi[q] / (1.f - pi[q] + eps);
+        out[q] = coef * coef * acc;
+      }
+    }
+  }
+}
+
 // grid (H).  Dynamic smem (floats): qb[na*d], ob[na*d], pi[na*M], key[na*M], x[na*M], G[M],
-// with candidate sets Gc[M], then e[kHeadWarps*d] (Gram scratch); with candidate sets the
+// with candidate sets Gc[M], then with a Gram matrix its staged columns; with candidate sets the
 // membership bytes cm[na*M]; then kb[M*d], vb[M*d] (this head's means, staged).
 __global__ void __launch_bounds__(kHeadThreads) k_head(const __grid_constant__ HeadArgs a) {
   extern __shared__ float sm[];
@@ -413,13 +496,14 @@ __global__ void __launch_bounds__(kHeadThreads) k_head(const __grid_constant__ H
   float* x = key + na * M;
   float* G = x + na * M;
   float* Gc = G + M;                         // best-response keys restricted to C_i
-  float* ew = Gc + (restricted ? M : 0);
-  uint8_t* cm = reinterpret_cast<uint8_t*>(ew + kHeadWarps * d);
+  float* gs = Gc + (restricted ? M : 0);     // staged columns of the Gram matrix
+  float* state_end = gs + (a.gram ? gram_stage_bytes(d) / sizeof(float) : 0);
+  uint8_t* cm = reinterpret_cast<uint8_t*>(state_end);
   // float4 stores below: the staged means start on a 16-byte boundary
   const size_t cm_bytes = restricted ? (((size_t)na * M + 15) & ~(size_t)15) : 0;
   float* kb_s = reinterpret_cast<float*>(
       reinterpret_cast<uint8_t*>(sm) +
-      (((reinterpret_cast<uint8_t*>(ew + kHeadWarps * d) - reinterpret_cast<uint8_t*>(sm)) + 15) & ~(ptrdiff_t)15) +
+      (((reinterpret_cast<uint8_t*>(state_end) - reinterpret_cast<uint8_t*>(sm)) + 15) & ~(ptrdiff_t)15) +
       cm_bytes);
   float* vb_s = kb_s + (size_t)M * d;
   launch_dependents();
@@ -539,26 +623,9 @@ __global__ void __launch_bounds__(kHeadThreads) k_head(const __grid_constant__ H
     }
     __syncthreads();
   } else if (a.mode == CAST_ROUTE_OMISSION) {
-    float* e = ew + warp * d;
-    for (int p = warp; p < na * M; p += kHeadWarps) {
-      const int i = p / M, m = p - i * M;
-      const float* vm = vb + (int64_t)m * kv_stride;
-      const float coef = pi[p] / (1.f - pi[p] + a.eps);
-      float acc = 0.f;
-      {
-        for (int c = lane; c < d; c += 32) e[c] = ob[i * d + c] - vm[c];
-        __syncwarp();
-        const float* Gm = a.gram + (int64_t)h * d * d;
-        for (int r = lane; r < d; r += 32) {
-          float y = 0.f;
-          for (int c = 0; c < d; ++c) y = fmaf(Gm[(int64_t)r * d + c], e[c], y);
-          acc = fmaf(e[r], y, acc);
-        }
-        __syncwarp();
-      }
-      acc = warp_sum(acc);
-      if (lane == 0) key[p] = coef * coef * acc;
-    }
+    const float* Gm = a.gram + (int64_t)h * d * d;
+    if (d == 128) gram_scores<128>(Gm, ob, vb, kv_stride, na, M, M, pi, a.eps, gs, key);
+    else gram_scores<64>(Gm, ob, vb, kv_stride, na, M, M, pi, a.eps, gs, key);
     __syncthreads();
   }
   if (a.u_out)
@@ -949,11 +1016,11 @@ __host__ __device__ inline uint32_t take_smem(size_t& o, size_t bytes) {
 // Byte offsets of the wide kernel's shared memory.  The o_bar partials of the warps share
 // their space with the rank-0 arrays, which are only written after the partials are reduced.
 struct WideLayout {
-  uint32_t qb, ob, obp, red, sl, pl, ew, coef, owp, u, x, sq, G, red2, hist, pre, cm;
+  uint32_t qb, ob, obp, red, sl, pl, gs, coef, owp, u, x, sq, G, red2, hist, pre, cm;
   size_t total;
 };
 __host__ __device__ inline WideLayout wide_layout(int na, int M, int d, int mr, bool refine,
-                                                  bool restricted) {
+                                                  bool restricted, bool gram) {
   WideLayout L{};
   size_t o = 0;
   const size_t naf = (size_t)na * sizeof(float);
@@ -963,7 +1030,7 @@ __host__ __device__ inline WideLayout wide_layout(int na, int M, int d, int mr, 
   L.red = take_smem(o, 2 * naf);
   L.sl = take_smem(o, naf * mr);
   L.pl = take_smem(o, naf * mr);
-  L.ew = take_smem(o, (size_t)kWideWarps * d * sizeof(float));
+  L.gs = take_smem(o, gram ? gram_stage_bytes(d) : 0);   // staged columns of the Gram matrix
   L.coef = take_smem(o, 3 * naf);
   const size_t region = o;
   L.owp = (uint32_t)region;
@@ -1125,14 +1192,13 @@ __global__ void __launch_bounds__(kWideThreads) k_head_wide(const __grid_constan
   const bool refine = a.passes > 0 && K > 0 && K < M;
   const int mr = (M + cl - 1) / cl;
   const int m0 = min(M, rank * mr), m1 = min(M, m0 + mr), nm = m1 - m0;
-  const WideLayout L = wide_layout(na, M, HD, mr, refine, restricted);
+  const WideLayout L = wide_layout(na, M, HD, mr, refine, restricted, a.gram != nullptr);
   float* qb = reinterpret_cast<float*>(wsm + L.qb);
   float* ob = reinterpret_cast<float*>(wsm + L.ob);
   float* obp = reinterpret_cast<float*>(wsm + L.obp);
   float* red = reinterpret_cast<float*>(wsm + L.red);
   float* sl = reinterpret_cast<float*>(wsm + L.sl);    // [na][mr] scores s of this CTA's blocks
   float* pl = reinterpret_cast<float*>(wsm + L.pl);    // [na][mr] pi, then the omission score u
-  float* ew = reinterpret_cast<float*>(wsm + L.ew);
   const float* kbar = a.kbar + h * HD;
   const float* vbar = a.vbar + h * HD;
   launch_dependents();
@@ -1283,27 +1349,8 @@ __global__ void __launch_bounds__(kWideThreads) k_head_wide(const __grid_constan
       }
     }
   } else if (a.mode == CAST_ROUTE_OMISSION) {
-    float* e = ew + warp * HD;
-    const float* Gm = a.gram + (int64_t)h * HD * HD;
-    for (int m = m0 + warp; m < m1; m += kWideWarps) {
-      for (int i = 0; i < na; ++i) {
-        for (int c = lane; c < HD; c += 32) e[c] = ob[i * HD + c] - vbar[(int64_t)m * D + c];
-        __syncwarp();
-        float acc = 0.f;
-        for (int r = lane; r < HD; r += 32) {
-          float y = 0.f;
-          for (int c = 0; c < HD; ++c) y = fmaf(Gm[(int64_t)r * HD + c], e[c], y);
-          acc = fmaf(e[r], y, acc);
-        }
-        __syncwarp();
-        acc = warp_sum(acc);
-        if (lane == 0) {
-          const int q = i * mr + (m - m0);
-          const float coef = pl[q] / (1.f - pl[q] + a.eps);
-          pl[q] = coef * coef * acc;
-        }
-      }
-    }
+    gram_scores<HD>(a.gram + (int64_t)h * HD * HD, ob, vbar + (int64_t)m0 * D, D, na, nm, mr, pl, a.eps,
+                    reinterpret_cast<float*>(wsm + L.gs), pl);
   }
   __syncthreads();
   // every CTA pushes its keys into rank 0's u[na][M] (that space held o_bar partials, which
@@ -1448,33 +1495,42 @@ __global__ void __launch_bounds__(kWideThreads) k_head_wide(const __grid_constan
   }
 }
 
-// shared state of the single-CTA head kernel without the staged means
-size_t head_state_bytes(const cast_route_args& a) {
+// The limits that choose and refuse a per-head kernel count limit_scratch() bytes of scratch
+// whether or not there is a Gram matrix; the launch takes what its layout needs (the Gram
+// matrix's staged columns, 16.5 KB at d = 128, or nothing).
+constexpr size_t kHeadSmemLimit = 200 * 1024;
+size_t limit_scratch(const cast_route_args& a) { return (size_t)kHeadWarps * a.d * sizeof(float); }
+size_t gram_bytes(const cast_route_args& a) { return a.gram ? gram_stage_bytes(a.d) : 0; }
+static_assert(kHeadSmemLimit + gram_stage_bytes(128) + 1024 <= 227 * 1024, "shared memory of one CTA");
+
+// shared memory of the single-CTA head kernel, which also holds k_bar and v_bar of its head
+size_t head_staged_bytes(const cast_route_args& a, size_t scratch) {
   const bool restricted = a.candidates != nullptr;
   const size_t floats = (size_t)2 * a.n_anchors * a.d + (size_t)3 * a.n_anchors * a.M + (size_t)a.M +
-                        (restricted ? (size_t)a.M : 0) + (size_t)kHeadWarps * a.d;
-  return floats * sizeof(float) + (restricted ? align_up((size_t)a.n_anchors * a.M, 16) : 0);
+                        (restricted ? (size_t)a.M : 0);
+  const size_t state =
+      floats * sizeof(float) + scratch + (restricted ? align_up((size_t)a.n_anchors * a.M, 16) : 0);
+  return align_up(state, 16) + (size_t)2 * a.M * a.d * sizeof(float);
 }
-
-constexpr size_t kHeadSmemLimit = 200 * 1024;
-// the single-CTA head kernel holds k_bar and v_bar of its head in shared memory
-size_t head_staged_bytes(const cast_route_args& a) {
-  return align_up(head_state_bytes(a), 16) + (size_t)2 * a.M * a.d * sizeof(float);
+bool head_stages_kv(const cast_route_args& a) {
+  return a.M <= 1024 && head_staged_bytes(a, limit_scratch(a)) <= kHeadSmemLimit;
 }
-bool head_stages_kv(const cast_route_args& a) { return a.M <= 1024 && head_staged_bytes(a) <= kHeadSmemLimit; }
 
 size_t wide_bytes(const cast_route_args& a) {
   const int K_eff = a.K < a.M ? a.K : a.M;
   const int cl = wide_cluster(a.M);
   const int mr = (a.M + cl - 1) / cl;
   return wide_layout(a.n_anchors, a.M, a.d, mr, a.refine_passes > 0 && K_eff > 0 && K_eff < a.M,
-                     a.candidates != nullptr).total;
+                     a.candidates != nullptr, a.gram != nullptr).total;
 }
 
 }  // namespace
 
+size_t route_head_limit_bytes(const cast_route_args& a) {
+  return head_stages_kv(a) ? head_staged_bytes(a, limit_scratch(a)) : wide_bytes(a) - gram_bytes(a) + limit_scratch(a);
+}
 size_t route_head_smem_bytes(const cast_route_args& a) {
-  return head_stages_kv(a) ? head_staged_bytes(a) : wide_bytes(a);
+  return head_stages_kv(a) ? head_staged_bytes(a, gram_bytes(a)) : wide_bytes(a);
 }
 
 size_t route_pool_smem_bytes(const cast_route_args& a) {
