@@ -62,7 +62,14 @@ __global__ void __launch_bounds__(kSumThreads) k_sumsq(const __grid_constant__ S
 #pragma unroll
     for (int u = 0; u < kUnroll; ++u) acc[u & 1] += v[u];
   }
-  for (; g < g1; g += kSumThreads) acc[0] += sumsq16(base + g * 16, a.elt);
+  // the last, partial round: its loads are in flight together too (one after another they cost
+  // a DRAM latency each: 7 of them, 5 of 19 us, for a 77 MB Matrix-Game-shaped call)
+  float v[kUnroll];
+#pragma unroll
+  for (int u = 0; u < kUnroll; ++u)
+    v[u] = g + (int64_t)u * kSumThreads < g1 ? sumsq16(base + (g + (int64_t)u * kSumThreads) * 16, a.elt) : 0.f;
+#pragma unroll
+  for (int u = 0; u < kUnroll; ++u) acc[0] += v[u];
   float s = acc[0] + acc[1];
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
@@ -92,6 +99,7 @@ struct SelectArgs {
 };
 
 constexpr int kSelectThreads = CAST_MAX_FRAMES;
+constexpr int kPartials = 40;   // splits of a frame whose sums are loaded at once
 
 __device__ __forceinline__ float block_min_max(float v, bool want_max, float* red) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -121,8 +129,15 @@ __global__ void __launch_bounds__(kSelectThreads) k_select(const __grid_constant
     float r = 0.f;
     if (live) {
       const float* p = a.partial + ((int64_t)k * N + i) * a.nsplit;
+      // summed in split order, kPartials loads in flight (a serial loop took 3 us a branch)
       float s = 0.f;
-      for (int q = 0; q < a.nsplit; ++q) s += p[q];
+      for (int q0 = 0; q0 < a.nsplit; q0 += kPartials) {
+        float v[kPartials];
+#pragma unroll
+        for (int q = 0; q < kPartials; ++q) v[q] = q0 + q < a.nsplit ? __ldcg(p + q0 + q) : 0.f;
+#pragma unroll
+        for (int q = 0; q < kPartials; ++q) s += v[q];
+      }
       r = sqrtf(s / (float)a.frame_elems);
       if (a.rms_out) a.rms_out[(int64_t)k * N + i] = r;
     }
