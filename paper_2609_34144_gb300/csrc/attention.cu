@@ -900,9 +900,7 @@ AttnPlan attention_plan(const cast_attn_args& a) {
   p.n_hist_tiles = hist_geom(a.hist).spatial ? (keff + 1) / 2 : keff * p.tiles_per_block;
   const int n_tiles = p.n_cur_tiles + p.n_hist_tiles;
   const int units = (p.n_pairs + p.n_single) * a.n_anchors * a.H;
-  int dev = 0, nsm = 148;
-  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-  if (nsm < 1) nsm = 1;
+  const int nsm = sm_count();
   // whole rounds of one unit per SM run unsplit; the units of the last, partial round are
   // split along K/V over the SMs (never into parts of fewer than 4 tiles)
   const int rounds = units / nsm;

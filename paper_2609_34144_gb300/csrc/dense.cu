@@ -384,8 +384,7 @@ int tile_columns(int row_pairs, int N, int n_k, int pairs) {
 
 cast_status gemm_anchor_rows(const AnchorGemm& g, cudaStream_t st) {
   if (g.n_anchors < 1 || g.S < 1 || g.N < 1 || g.K < 1) return CAST_OK;
-  int dev = 0, nsm = 148;
-  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  const int nsm = sm_count();
   const int pairs = nsm > 1 ? nsm / 2 : 1;
   GemmKArgs k{};
   k.S = g.S;

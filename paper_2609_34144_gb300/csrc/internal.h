@@ -40,6 +40,10 @@ bool once_per_device(std::atomic<uint64_t>& done, F&& setup) {
   return true;
 }
 
+// SMs of the current device (148 where there is none: plans are also sized without a GPU).  Asked
+// of the runtime once per device: the plans ask several times in every call.
+int sm_count();
+
 constexpr size_t kWsAlign = 256;
 inline size_t align_up(size_t x, size_t a = kWsAlign) { return (x + a - 1) / a * a; }
 

@@ -1053,8 +1053,7 @@ cast_status launch_kind(const CUtensorMap& tm, const CUtensorMap* tm_sw, const C
   if (k.img) {
     // bf16: the blend as tensor-core GEMMs over the matrices K_transport wrote
     // persistent: one CTA per SM over the (tile, 128-channel chunk) items of this kind
-    int dev = 0, nsm = 148;
-    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    const int nsm = sm_count();
     const int items = ((k.C + kTbNC - 1) / kTbNC) * n_tiles;
     cudaLaunchConfig_t bc{};
     bc.gridDim = dim3(items < nsm ? items : nsm, 1, 1);
@@ -1161,9 +1160,7 @@ ParPlan par_plan(const cast_par_args& a) {
   // run concurrently on the side stream; each segment re-reads its first anchor.  Measured at
   // the Matrix-Game size (3 pairs: full tiles 2 segments, 0.049 ms against 0.053 ms with 3)
   // and the PAR sweep (edge tiles 3 segments, 2 % faster than 2).
-  int dev = 0, nsm = 148;
-  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-  if (nsm <= 0) nsm = 148;
+  const int nsm = sm_count();
   auto segs = [&](int n_tiles, int depth) {
     const int want_ctas = depth * nsm;
     const int per_seg = n_tiles * p.n_chunk;
@@ -1181,6 +1178,32 @@ ParPlan par_plan(const cast_par_args& a) {
   p.total_bytes = p.n_target > 0 ? p.rec_bytes + p.trans_bytes + p.img_bytes : 0;
   return p;
 }
+
+namespace {
+struct FastSrc {
+  signed char v[kNV];
+};
+FastSrc make_fast_src() {
+  FastSrc f{};
+  // record entry t = 3 * bin + comp of an 8x8 tile from the 96 reduced values (+ W at DC = 96)
+  int pos[40 * 4];
+  for (int q = 0; q < 160; ++q) pos[q] = -1;
+  for (int n = 0; n < 96; ++n) pos[fast_value(n)] = n;
+  for (int t = 0; t < kNV; ++t) {
+    const int b = t / 3, comp = t % 3, ky = b / 5, kx = b % 5;
+    const bool edge = kx == 0 || kx == 4;
+    const bool selfc = edge && (ky == 0 || ky == 4);
+    const bool mirror = edge && !selfc && ky > 4;
+    const int r = mirror ? (8 - ky) * 5 + kx : b;
+    int src = 0;
+    if (r == 0) src = comp == 2 ? 96 + 1 : 0;                 // DC: only W
+    else if (comp == 1 && selfc) src = 0;                     // Im Z of a real bin
+    else src = (pos[r * 4 + comp] + 1) * ((mirror && comp == 1) ? -1 : 1);
+    f.v[t] = (signed char)src;
+  }
+  return f;
+}
+}  // namespace
 
 cast_status launch_par(const cast_par_args& a, void* ws, cudaStream_t st) {
   const ParPlan p = par_plan(a);
@@ -1237,24 +1260,8 @@ cast_status launch_par(const cast_par_args& a, void* ws, cudaStream_t st) {
   k.band = pp.band_radius;
   k.gate_mode = pp.gate_mode;
   k.wait_ns = 2000000000ull;
-  {
-    // record entry t = 3 * bin + comp of an 8x8 tile from the 96 reduced values (+ W at DC = 96)
-    int pos[40 * 4];
-    for (int q = 0; q < 160; ++q) pos[q] = -1;
-    for (int n = 0; n < 96; ++n) pos[fast_value(n)] = n;
-    for (int t = 0; t < kNV; ++t) {
-      const int b = t / 3, comp = t % 3, ky = b / 5, kx = b % 5;
-      const bool edge = kx == 0 || kx == 4;
-      const bool selfc = edge && (ky == 0 || ky == 4);
-      const bool mirror = edge && !selfc && ky > 4;
-      const int r = mirror ? (8 - ky) * 5 + kx : b;
-      int src = 0;
-      if (r == 0) src = comp == 2 ? 96 + 1 : 0;                 // DC: only W
-      else if (comp == 1 && selfc) src = 0;                     // Im Z of a real bin
-      else src = (pos[r * 4 + comp] + 1) * ((mirror && comp == 1) ? -1 : 1);
-      k.fast_src[t] = (signed char)src;
-    }
-  }
+  static const FastSrc fast_src = make_fast_src();
+  std::copy(fast_src.v, fast_src.v + kNV, k.fast_src);
 
   CUtensorMap tm;
   if (!make_r_map(&tm, a, p.chunk)) return fail(CAST_ERR_CUDA, "PAR: cuTensorMapEncodeTiled failed");

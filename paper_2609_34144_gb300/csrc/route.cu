@@ -1544,9 +1544,7 @@ RoutePlan route_plan(const cast_route_args& a) {
   p.n_seg = a.n_anchors + 2 * a.M;
   // per launch (anchor frames, history blocks): a cluster of up to 8 CTAs per segment, enough
   // CTAs to cover the SMs a few times, each streaming >= 64 rows
-  int dev = 0, nsm = 148;
-  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-  const int target = 4 * (nsm > 0 ? nsm : 148);
+  const int target = 4 * sm_count();
   auto splits = [&](int n_seg, int rows) {
     int ns = n_seg > 0 ? (target + n_seg - 1) / n_seg : 1;
     if (ns > kMaxClusterSplit) ns = kMaxClusterSplit;
@@ -1594,6 +1592,24 @@ cast_status launch_route(const cast_route_args& a, void* ws, cudaStream_t st) {
   pa.nbx = hg.nbx;
   for (int k = 0; k < a.n_anchors; ++k) pa.anchors[k] = a.anchors[k];
 
+  // every kernel may take what the limits of validation allow it (set once per device)
+  static std::atomic<uint64_t> attr_done{0};
+  if (!once_per_device(attr_done, [] {
+        auto allow = [](const void* fn) {
+          cudaFuncAttributes fa{};
+          if (cudaFuncGetAttributes(&fa, fn) != cudaSuccess) return false;
+          return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      227 * 1024 - (int)fa.sharedSizeBytes) == cudaSuccess;
+        };
+        using b16 = __nv_bfloat16;
+        return allow((const void*)k_pool<b16, false, true>) && allow((const void*)k_pool<b16, true, false>) &&
+               allow((const void*)k_pool<b16, false, false>) && allow((const void*)k_pool<float, false, true>) &&
+               allow((const void*)k_pool<float, true, false>) && allow((const void*)k_pool<float, false, false>) &&
+               allow((const void*)k_head) && allow((const void*)k_head_small<64>) &&
+               allow((const void*)k_head_small<128>) && allow((const void*)k_head_wide<64>) &&
+               allow((const void*)k_head_wide<128>);
+      }))
+    return check_launch("routing kernel attributes");
   const size_t psm = route_pool_smem_bytes(a);
   const PoolShape ps = pool_shape(D, pa.elt);
   const int row_bytes = D * pa.elt;
@@ -1620,9 +1636,6 @@ cast_status launch_route(const cast_route_args& a, void* ws, cudaStream_t st) {
                 : (hist && hg.spatial ? k_pool<__nv_bfloat16, true, false> : k_pool<__nv_bfloat16, false, false>);
     else
       fn = bulk ? k_pool<float, false, true> : (hist && hg.spatial ? k_pool<float, true, false> : k_pool<float, false, false>);
-    if (smem > 48 * 1024 &&
-        cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-      return fail(CAST_ERR_CUDA, "routing: cannot reserve %zu B of shared memory for pooling", smem);
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(nsplit, hist ? 2 * a.M : a.n_anchors, 1);
     cfg.blockDim = dim3(ps.cgs * ps.lanes_r, 1, 1);
@@ -1702,9 +1715,6 @@ cast_status launch_route(const cast_route_args& a, void* ws, cudaStream_t st) {
   const size_t hsm = small ? small_head_bytes(a) : route_head_smem_bytes(a);
   auto head_fn = small ? (a.d == 128 ? k_head_small<128> : k_head_small<64>)
                        : !p.wide ? k_head : (a.d == 128 ? k_head_wide<128> : k_head_wide<64>);
-  if (hsm > 48 * 1024 &&
-      cudaFuncSetAttribute(head_fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)hsm) != cudaSuccess)
-    return fail(CAST_ERR_CUDA, "routing: cannot reserve %zu B of shared memory", hsm);
   cudaLaunchConfig_t hc{};
   hc.gridDim = p.wide ? dim3(p.cl, a.H, 1) : dim3(a.H, 1, 1);
   hc.blockDim = dim3(p.wide ? kWideThreads : kHeadThreads, 1, 1);

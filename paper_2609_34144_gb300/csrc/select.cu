@@ -182,10 +182,8 @@ __global__ void __launch_bounds__(kSelectThreads) k_select(const __grid_constant
 
 int sum_splits(const cast_select_args& a) {
   const int64_t groups = a.frame_elems * (a.dtype == CAST_BF16 ? 2 : 4) / 16;
-  int dev = 0, nsm = 148;
-  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   const int units = a.n_branch * a.n_frames;
-  int nsplit = (4 * (nsm > 0 ? nsm : 148) + units - 1) / (units > 0 ? units : 1);
+  int nsplit = (4 * sm_count() + units - 1) / (units > 0 ? units : 1);
   // at least 64 KB per CTA
   const int64_t max_split = groups / 4096 > 0 ? groups / 4096 : 1;
   if (nsplit > max_split) nsplit = (int)max_split;

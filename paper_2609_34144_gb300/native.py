@@ -8,6 +8,7 @@ is no fallback: without the built library, importing this module raises.
 from __future__ import annotations
 
 import ctypes as C
+import math
 import os
 
 import torch
@@ -146,13 +147,20 @@ def _check(status):
         raise CastError(status, _lib.cast_last_error_detail().decode())
 
 
+# The calls below marshal in as few Python steps as they can: structures are filled by position,
+# pointers are plain integers, a tensor's shape and strides are read once and the workspace is
+# sized only where the caller brought none.  A call on a small chunk is bound by this path
+# (attention of 5 frames of 13x27: 29 us of host time around 17 us of GPU work before).
 def _ptr(t):
-    return None if t is None else C.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
+
+
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream",
+                      lambda dev: torch.cuda.current_stream(dev).cuda_stream)
 
 
 def _stream(stream=None):
-    s = torch.cuda.current_stream() if stream is None else stream
-    return C.c_void_p(s.cuda_stream)
+    return _raw_stream(torch.cuda.current_device()) if stream is None else stream.cuda_stream
 
 
 def _dtype_code(t):
@@ -164,35 +172,39 @@ def _dtype_code(t):
 
 
 def _host_i32(seq):
-    arr = (_i32 * max(1, len(seq)))(*[int(v) for v in seq])
-    return arr
+    return (_i32 * max(1, len(seq)))(*map(int, seq))
 
 
 def _row_stride(t):
     """Token row stride (elements) of a [frames|blocks, tokens, H, d] tensor whose H, d are
     contiguous and whose tokens of a frame are evenly spaced."""
-    if t.dim() != 4 or t.stride(3) != 1 or t.stride(2) != t.shape[3]:
+    sh, st = t.shape, t.stride()
+    if len(sh) != 4 or st[3] != 1 or st[2] != sh[3]:
         raise ValueError("expected [N, T, H, d] with contiguous (H, d)")
-    if t.shape[0] > 1 and t.stride(0) != t.stride(1) * t.shape[1]:
+    if sh[0] > 1 and st[0] != st[1] * sh[1]:
         raise ValueError("frames must be consecutive token rows")
-    return t.stride(1)
+    return st[1]
+
+
+_BLOCKS = HistLayout()   # copied into the argument structures, never changed
 
 
 def _history(k_hist, H, d):
     """(M, B_v, row stride, HistLayout) of the history tensor: [M, B_v, H, d] blocks, or
     [frames, Hg, Wg, H, d] frames cut into (1, 8, 8) blocks (M = frames ceil(Hg/8) ceil(Wg/8),
     nominal B_v = 64); None means no history."""
-    lay = HistLayout()
     if k_hist is None or k_hist.shape[0] == 0:
-        return 0, 0, H * d, lay
+        return 0, 0, H * d, _BLOCKS
     if k_hist.dim() == 5:
+        lay = HistLayout()
         F, Hg, Wg = k_hist.shape[:3]
         if Hg > 1 and k_hist.stride(1) != k_hist.stride(2) * Wg:
             raise ValueError("history frames must hold consecutive token rows")
         rs = _row_stride(k_hist.flatten(1, 2))
         lay.kind, lay.frames, lay.Hg, lay.Wg = HIST_FRAMES, F, Hg, Wg
         return F * (-(-Hg // 8)) * (-(-Wg // 8)), 64, rs, lay
-    return k_hist.shape[0], k_hist.shape[1], _row_stride(k_hist), lay
+    rs = _row_stride(k_hist)
+    return k_hist.shape[0], k_hist.shape[1], rs, _BLOCKS
 
 
 def _workspace(nbytes, device):
@@ -217,6 +229,7 @@ def default_par_params():
 
 
 # --------------------------------------------------------------------------- routing
+_NO_REFINE = dict(passes=0, lambda_anc=0.0, lambda_rec=0.0, tol=0.0)
 REFINE_PAPER = dict(passes=2, lambda_anc=1.0, lambda_rec=1.0, tol=1e-6)   # Tab. config_cast
 
 
@@ -233,19 +246,11 @@ def _route_args(q, anchors, k_hist, v_hist, K, gram=None, eps=1e-8, mode=ROUTE_O
                 refine=None, candidates=None):
     N, S, H, d = q.shape
     M, B_v, rs, lay = _history(k_hist, H, d)
-    a = RouteArgs()
-    a.q, a.q_row_stride = _ptr(q), _row_stride(q)
-    a.n_frames, a.S, a.H, a.d = N, S, H, d
-    a.dtype = _dtype_code(q)
-    a._anchors = _host_i32(anchors)
-    a.anchors = C.cast(a._anchors, C.POINTER(_i32))
-    a.n_anchors = len(anchors)
-    a.k_hist, a.v_hist = _ptr(k_hist), _ptr(v_hist)
-    a.hist_row_stride = rs
-    a.M, a.B_v, a.hist = M, B_v if M > 0 else k_hist.shape[1], lay
-    a.gram = _ptr(gram)
-    a.K, a.eps, a.mode = K, eps, mode
-    a.candidates, a.M_c = _candidates(candidates)
+    a = RouteArgs(q.data_ptr(), _row_stride(q), N, S, H, d, _dtype_code(q), _host_i32(anchors), len(anchors),
+                  _ptr(k_hist), _ptr(v_hist), rs, M, B_v if M > 0 else k_hist.shape[1], _ptr(gram), K, eps, mode)
+    a.hist = lay
+    if candidates is not None:
+        a.candidates, a.M_c = _candidates(candidates)
     if refine:
         a.refine_passes, a.lambda_anc = refine["passes"], refine["lambda_anc"]
         a.lambda_rec, a.refine_tol = refine["lambda_rec"], refine["tol"]
@@ -275,10 +280,7 @@ def cast_route_topk(q, anchors, k_hist, v_hist, K, gram=None, eps=1e-8, mode=ROU
         kb = torch.empty((M, H, d), dtype=torch.float32, device=dev)
         vb = torch.empty((M, H, d), dtype=torch.float32, device=dev)
     a.idx, a.u, a.qbar, a.kbar, a.vbar = _ptr(idx), _ptr(u), _ptr(qb), _ptr(kb), _ptr(vb)
-    keff_out = _i32(0)
-    a.k_eff = C.pointer(keff_out)
-    need = _lib.cast_route_workspace_size(C.byref(a))
-    ws = workspace if workspace is not None else _workspace(need, dev)
+    ws = workspace if workspace is not None else _workspace(_lib.cast_route_workspace_size(C.byref(a)), dev)
     _check(_lib.cast_route_topk(C.byref(a), _ptr(ws), ws.numel(), _stream(stream)))
     out = [idx]
     if want_u:
@@ -305,19 +307,10 @@ def cast_route_topk_noalloc(q, anchors, k_hist, v_hist, K, gram=None, eps=1e-8,
 def _attn_args(q, k_cur, v_cur, anchors, k_hist, v_hist, idx, scale=0.0):
     N, S, H, d = q.shape
     M, B_v, rs, lay = _history(k_hist, H, d)
-    a = AttnArgs()
-    a.q, a.k_cur, a.v_cur = _ptr(q), _ptr(k_cur), _ptr(v_cur)
-    a.q_row_stride, a.cur_row_stride = _row_stride(q), _row_stride(k_cur)
-    a.n_frames, a.S, a.H, a.d = N, S, H, d
-    a._anchors = _host_i32(anchors)
-    a.anchors = C.cast(a._anchors, C.POINTER(_i32))
-    a.n_anchors = len(anchors)
-    a.k_hist, a.v_hist = _ptr(k_hist), _ptr(v_hist)
-    a.hist_row_stride = rs
-    a.M, a.B_v, a.hist = M, B_v, lay
-    a.idx = _ptr(idx)
-    a.K_eff = idx.shape[-1] if idx is not None else 0
-    a.scale = scale
+    a = AttnArgs(q.data_ptr(), k_cur.data_ptr(), _ptr(v_cur), _row_stride(q), _row_stride(k_cur), N, S, H, d,
+                 _host_i32(anchors), len(anchors), _ptr(k_hist), _ptr(v_hist), rs, M, B_v, _ptr(idx),
+                 idx.shape[-1] if idx is not None else 0, scale)
+    a.hist = lay
     return a
 
 
@@ -330,15 +323,13 @@ def cast_anchor_attention(q, k_cur, v_cur, anchors, k_hist, v_hist, idx, scale=0
                           out_dtype=torch.bfloat16, want_lse=False, out=None, workspace=None,
                           stream=None):
     """Returns O [K_f, S, H*d] (and lse [K_f, H, S])."""
-    N, S, H, d = q.shape
-    Kf = len(anchors)
     a = _attn_args(q, k_cur, v_cur, anchors, k_hist, v_hist, idx, scale)
+    Kf, S, H, d = len(anchors), a.S, a.H, a.d
     o = out if out is not None else torch.empty((Kf, S, H * d), dtype=out_dtype, device=q.device)
     a.o, a.o_dtype = _ptr(o), _dtype_code(o)
     lse = torch.empty((Kf, H, S), dtype=torch.float32, device=q.device) if want_lse else None
     a.lse = _ptr(lse)
-    need = _lib.cast_attention_workspace_size(C.byref(a))
-    ws = workspace if workspace is not None else _workspace(need, q.device)
+    ws = workspace if workspace is not None else _workspace(_lib.cast_attention_workspace_size(C.byref(a)), q.device)
     _check(_lib.cast_anchor_attention(C.byref(a), _ptr(ws), ws.numel(), _stream(stream)))
     return (o, lse) if want_lse else o
 
@@ -346,14 +337,9 @@ def cast_anchor_attention(q, k_cur, v_cur, anchors, k_hist, v_hist, idx, scale=0
 # --------------------------------------------------------------------------- PAR
 def _par_args(r, anchor_mask, channel_weight=None, params=None):
     F, Hg, Wg, Cc = r.shape
-    a = ParArgs()
-    a.r, a.dtype = _ptr(r), _dtype_code(r)
-    a.F, a.Hg, a.Wg, a.C = F, Hg, Wg, Cc
-    a._mask = (C.c_uint8 * F)(*[1 if m else 0 for m in anchor_mask])
-    a.anchor_mask = C.cast(a._mask, C.POINTER(C.c_uint8))
-    a.channel_weight = _ptr(channel_weight)
-    a.params = params if params is not None else default_par_params()
-    return a
+    return ParArgs(r.data_ptr(), _dtype_code(r), F, Hg, Wg, Cc,
+                   (C.c_uint8 * F)(*[1 if m else 0 for m in anchor_mask]), _ptr(channel_weight),
+                   params if params is not None else default_par_params())
 
 
 def par_workspace_size(r, anchor_mask, params=None):
@@ -367,8 +353,7 @@ def cast_par_reconstruct(r, anchor_mask, channel_weight=None, params=None, works
     if not r.is_contiguous():
         raise ValueError("r must be contiguous [F, Hg, Wg, C]")
     a = _par_args(r, anchor_mask, channel_weight, params)
-    need = _lib.cast_par_workspace_size(C.byref(a))
-    ws = workspace if workspace is not None else _workspace(need, r.device)
+    ws = workspace if workspace is not None else _workspace(_lib.cast_par_workspace_size(C.byref(a)), r.device)
     _check(_lib.cast_par_reconstruct(C.byref(a), _ptr(ws), ws.numel(), _stream(stream)))
     return r
 
@@ -379,27 +364,14 @@ def block_args(q, k_cur, v_cur, anchors, k_hist, v_hist, K, grid, r_out, x=None,
                channel_weight=None, params=None, refine=None, w_o=None, b_o=None, candidates=None):
     N, S, H, d = q.shape
     M, B_v, rs, lay = _history(k_hist, H, d)
-    a = BlockArgs()
-    a.q, a.k_cur, a.v_cur = _ptr(q), _ptr(k_cur), _ptr(v_cur)
-    a.q_row_stride, a.cur_row_stride = _row_stride(q), _row_stride(k_cur)
-    a.n_frames, a.Hg, a.Wg, a.H, a.d = N, grid[0], grid[1], H, d
-    a._anchors = _host_i32(anchors)
-    a.anchors = C.cast(a._anchors, C.POINTER(_i32))
-    a.n_anchors = len(anchors)
-    a.k_hist, a.v_hist = _ptr(k_hist), _ptr(v_hist)
-    a.hist_row_stride = rs
-    a.M, a.B_v, a.hist = M, B_v if M > 0 else k_hist.shape[1], lay
-    a.gram, a.K, a.route_eps, a.route_mode, a.scale = _ptr(gram), K, route_eps, route_mode, scale
-    if refine:
-        a.route_refine_passes, a.route_lambda_anc = refine["passes"], refine["lambda_anc"]
-        a.route_lambda_rec, a.route_refine_tol = refine["lambda_rec"], refine["tol"]
-    a.r_out, a.r_dtype = _ptr(r_out), _dtype_code(r_out)
-    a.x = _ptr(x)
-    a.idx_out = _ptr(idx_out)
-    a.channel_weight = _ptr(channel_weight)
-    a.par = params if params is not None else default_par_params()
-    a.w_o, a.b_o = _ptr(w_o), _ptr(b_o)
-    a.route_candidates, a.route_M_c = _candidates(candidates)
+    refine = refine or _NO_REFINE
+    cand, M_c = _candidates(candidates)
+    a = BlockArgs(q.data_ptr(), k_cur.data_ptr(), _ptr(v_cur), _row_stride(q), _row_stride(k_cur), N, grid[0],
+                  grid[1], H, d, _host_i32(anchors), len(anchors), _ptr(k_hist), _ptr(v_hist), rs, M,
+                  B_v if M > 0 else k_hist.shape[1], _ptr(gram), K, route_eps, route_mode, refine["passes"],
+                  refine["lambda_anc"], refine["lambda_rec"], refine["tol"], scale, r_out.data_ptr(),
+                  _dtype_code(r_out), _ptr(x), _ptr(idx_out), _ptr(channel_weight),
+                  params if params is not None else default_par_params(), _ptr(w_o), _ptr(b_o), lay, cand, M_c)
     a._keep = (candidates,)
     return a
 
@@ -416,8 +388,7 @@ def cast_block_step(q, k_cur, v_cur, anchors, k_hist, v_hist, K, grid, r_out, x=
                     idx_out=None, workspace=None, stream=None, **kw):
     """route -> attention -> PAR at one attention residual site; fills r_out [N, S, H*d]."""
     a = block_args(q, k_cur, v_cur, anchors, k_hist, v_hist, K, grid, r_out, x, idx_out, **kw)
-    need = block_workspace_size(a)
-    ws = workspace if workspace is not None else _workspace(need, q.device)
+    ws = workspace if workspace is not None else _workspace(block_workspace_size(a), q.device)
     cast_block_step_args(a, ws, stream)
     return r_out
 
@@ -443,19 +414,14 @@ def library():
 def select_args(deltas, ages, anchor_mask, K_f, lambda_cov=0.5, eps=1e-8):
     """deltas: list of 0..2 device tensors [N_cur, ...] (same dtype, contiguous); ages int32 and
     anchor_mask uint8 device tensors [N_cur]."""
-    a = SelectArgs()
     N = ages.shape[0]
-    a.n_branch = len(deltas)
-    for k, dk in enumerate(deltas):
+    for dk in deltas:
         if not dk.is_contiguous():
             raise ValueError("control updates must be contiguous")
-        a.delta[k] = dk.data_ptr()
-    a.dtype = (F32 if deltas[0].dtype == torch.float32 else BF16) if deltas else F32
-    a.n_frames = N
-    a.frame_elems = deltas[0][0].numel() if deltas else 0
-    a.ages, a.anchor_mask = _ptr(ages), _ptr(anchor_mask)
-    a.K_f, a.lambda_cov, a.eps = K_f, lambda_cov, eps
-    return a
+    d0 = deltas[0] if deltas else None
+    return SelectArgs((_vp * 2)(*[dk.data_ptr() for dk in deltas]), len(deltas),
+                      BF16 if deltas and d0.dtype != torch.float32 else F32, N,
+                      math.prod(d0.shape[1:]) if deltas else 0, _ptr(ages), _ptr(anchor_mask), K_f, lambda_cov, eps)
 
 
 def cast_select_frames(deltas, ages, anchor_mask, K_f, lambda_cov=0.5, eps=1e-8, want_rms=False,
@@ -472,8 +438,7 @@ def cast_select_frames(deltas, ages, anchor_mask, K_f, lambda_cov=0.5, eps=1e-8,
     score = torch.empty(N, dtype=torch.float32, device=dev) if want_score else None
     a.ages_out, a.anchors_out, a.mask_out = _ptr(ages_out), _ptr(anchors), _ptr(mask)
     a.rms_out, a.score_out = _ptr(rms), _ptr(score)
-    need = _lib.cast_select_workspace_size(C.byref(a))
-    ws = workspace if workspace is not None else _workspace(need, dev)
+    ws = workspace if workspace is not None else _workspace(_lib.cast_select_workspace_size(C.byref(a)), dev)
     _check(_lib.cast_select_frames(C.byref(a), _ptr(ws), ws.numel(), _stream(stream)))
     out = [anchors, ages_out, mask]
     if want_rms:
@@ -492,26 +457,17 @@ def ffn_args(x, anchors, w1, b1, w2, b2, grid, r_out, channel_weight=None, param
     """x bf16 [F, S, D] (token rows contiguous per frame); w1 bf16 [D_ff, D], w2 bf16 [D, D_ff];
     b1 bf16 [D_ff] or None; b2 [D] of r_out's dtype or None; r_out [F, S, D] f32 or bf16."""
     F, S, D = x.shape[0], x.shape[1], x.shape[-1]
-    a = FfnArgs()
-    a.x, a.x_row_stride = _ptr(x), x.stride(1) if x.dim() == 3 else D
-    a.n_frames, a.Hg, a.Wg, a.D, a.D_ff = F, grid[0], grid[1], D, w1.shape[0]
-    a._anchors = _host_i32(anchors)
-    a.anchors = C.cast(a._anchors, C.POINTER(_i32))
-    a.n_anchors = len(anchors)
-    a.w1, a.b1, a.w2, a.b2 = _ptr(w1), _ptr(b1), _ptr(w2), _ptr(b2)
-    a.r_out = _ptr(r_out)
-    a.r_dtype = F32 if r_out.dtype == torch.float32 else BF16
-    a.channel_weight = _ptr(channel_weight)
-    a.par = params if params is not None else default_par_params()
-    return a
+    return FfnArgs(x.data_ptr(), x.stride(1) if x.dim() == 3 else D, F, grid[0], grid[1], D, w1.shape[0],
+                   _host_i32(anchors), len(anchors), w1.data_ptr(), _ptr(b1), _ptr(w2), _ptr(b2),
+                   r_out.data_ptr(), F32 if r_out.dtype == torch.float32 else BF16, _ptr(channel_weight),
+                   params if params is not None else default_par_params())
 
 
 def cast_ffn_step(x, anchors, w1, b1, w2, b2, grid, r_out, channel_weight=None, params=None,
                   workspace=None, stream=None):
     """Anchor FFN residuals into r_out's anchor rows, PAR for the skipped rows."""
     a = ffn_args(x, anchors, w1, b1, w2, b2, grid, r_out, channel_weight, params)
-    need = _lib.cast_ffn_workspace_size(C.byref(a))
-    ws = workspace if workspace is not None else _workspace(need, x.device)
+    ws = workspace if workspace is not None else _workspace(_lib.cast_ffn_workspace_size(C.byref(a)), x.device)
     _check(_lib.cast_ffn_step(C.byref(a), _ptr(ws), ws.numel(), _stream(stream)))
     return r_out
 
