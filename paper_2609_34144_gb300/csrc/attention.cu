@@ -285,6 +285,12 @@ __global__ void __launch_bounds__(kThreads, 1)
   tc_fence_after();
   const uint32_t tmem = bars->tmem_base;
   const uint64_t lim = a.wait_ns;
+  // Whether a converged warp's wait has gone on for too long (its deadline starts at the first call)
+  auto expired = [&](uint64_t& t0) -> bool {
+    const uint64_t now = global_ns();
+    if (t0 == 0) t0 = now;
+    return __any_sync(0xffffffffu, aborted(bars) || now - t0 > lim);
+  };
 
   if (warp < 4) {
   setmaxnreg_dec<kRegsCtl>();
@@ -383,10 +389,10 @@ __global__ void __launch_bounds__(kThreads, 1)
       uint64_t* const b = lane < 16 ? b0 : b1;
       const uint32_t par = (uint32_t)(lane < 16 ? ph0 : ph1) & 1u;
       if (__all_sync(0xffffffffu, mbar_try_wait(b, par))) return true;
-      const uint64_t t_begin = global_ns();
+      uint64_t t0 = 0;
       for (uint32_t it = 1;; ++it) {
         if (__all_sync(0xffffffffu, mbar_try_wait(b, par))) return true;
-        if ((it & 63u) == 0u && __any_sync(0xffffffffu, aborted(bars) || global_ns() - t_begin > lim)) return false;
+        if (it % kWaitTries == 0 && expired(t0)) return false;
       }
     };
     auto wait = [&](uint64_t* bar, int phase) -> bool { return wait2(bar, phase, bar, phase); };
@@ -517,10 +523,10 @@ __global__ void __launch_bounds__(kThreads, 1)
     // A phase of one barrier for the whole warp: one test in the usual case
     auto warp_wait = [&](uint64_t* bar, uint32_t parity) -> bool {
       if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
-      const uint64_t t_begin = global_ns();
+      uint64_t t0 = 0;
       for (uint32_t it = 1;; ++it) {
         if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
-        if ((it & 63u) == 0u && __any_sync(0xffffffffu, aborted(bars) || global_ns() - t_begin > lim)) return false;
+        if (it % kWaitTries == 0 && expired(t0)) return false;
       }
     };
     // K/V tile of the current history block (counted, so that no division sits in the loop)

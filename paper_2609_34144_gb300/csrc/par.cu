@@ -1,31 +1,37 @@
 // Phase-Aware Reconstruction of skipped frames (Section 4.3, Eqs. cross, confidence, gate,
-// fcpasm; App. A.2) in three passes per tile kind (full 8x8 tiles / truncated edge tiles):
+// fcpasm; App. A.2).  On every tile: the anchors' spectra, the channel-pooled
+//   Z = sum_c w_c F_b conj(F_a),  W = sum_c w_c |F_b||F_a|
+// of each anchor pair, from them reliability, phases theta, confidence and gate g (the transport),
+// and R_t = IRFFT2((1-alpha) F_a e^{i g alpha theta} + alpha F_b e^{-i g (1-alpha) theta}).
 //
+// bf16 residuals: two launches over every tile, on the tensor cores.
+//   K_stats_tc (tile, pair, chunk range): the transforms as one GEMM with the tile's DFT matrix per
+//       128-channel chunk, Z and W summed over channels into one record in the workspace.
+//   K_blend_tc (tile, targets of a pair, chunk range): the transport from the records, then the
+//       blend: on one tile, Eq. (fcpasm) is exactly two circular convolutions,
+//         R_t = h_a (*) R_a + h_b (*) R_b,  h = IDFT2 of the Hermitian-extended phasors
+//         phi_a = (1-alpha) e^{i g alpha theta}, phi_b = alpha e^{-i g (1-alpha) theta},
+//       so one UMMA chain per pair of targets computes [H_t1 ; H_t2] [X_a ; X_b] for 128 channels.
+//   Measured (GB300, 16 frames of 44x80 x 3072, 5 anchors): 160 -> 109 us against three launches
+//   per tile kind (register transforms, a transport that wrote the matrices, a blend that loaded
+//   them for every tile and chunk; edge tiles on a second stream).
+//
+// f32 residuals: three passes per tile kind (full 8x8 tiles / truncated edge tiles).
 //   K_stats (tile, channel chunk): one thread per channel streams the anchors of the tile in
 //       time order through a TMA 4-D map ([frame][row][col][channel], out-of-range rows/cols/
 //       channels arrive as zeros), forms each tile spectrum in registers (the previous anchor's
-//       spectrum stays in shared memory) and, for every anchor pair with targets, reduces
-//       Z = sum_c w_c F_b conj(F_a) and W = sum_c w_c |F_b||F_a| over the chunk's channels
-//       (warp transpose reductions) into one record in the workspace.
-//   K_transport (tile, pair[, target]): sums the records of the tile's channel chunks in chunk
-//       order (deterministic) and derives eta, reliability, principal phases, the confidence c
-//       and the gate g per bin; writes theta and g (and, for bf16, one target's blend matrix).
+//       spectrum stays in shared memory) and, for every anchor pair with targets, reduces Z and W
+//       over the chunk's channels (warp transpose reductions) into one record in the workspace.
+//   K_transport (tile, pair): sums the records of the tile's channel chunks in chunk order
+//       (deterministic) and writes theta and g.
 //   K_blend (tile, channel chunk): streams the anchors again (an L2 hit at these sizes), forms
-//       their spectra and writes every target straight from registers:
-//       R_t = IRFFT2((1-alpha) F_a e^{i g alpha theta} + alpha F_b e^{-i g (1-alpha) theta}).
-//       This is the f32 blend.  For bf16 residuals the blend runs on the tensor cores instead
-//       (K_blend_tc below): on one tile, Eq. (fcpasm) is exactly two circular convolutions,
-//         R_t = h_a (*) R_a + h_b (*) R_b,  h = IDFT2 of the Hermitian-extended phasors
-//         phi_a = (1-alpha) e^{i g alpha theta}, phi_b = alpha e^{-i g (1-alpha) theta},
-//       so K_transport also writes each target's 64 x 128 matrix [H_a | H_b] (two bf16 pieces,
-//       laid out as a swizzled UMMA operand) and one UMMA chain per pair of targets computes
-//       [H_t1 ; H_t2] [X_a ; X_b] for 128 channels (M = 128 output rows, K = 128 tokens).
+//       their spectra and writes every target straight from registers.
+// The passes are chained as programmatic dependents (the transport releases the blend at its
+// end), the full-tile chain on the caller's stream and the edge-tile chain on a second stream.
+//
 // The CTAs of a pass never wait on each other, so the passes fill the GPU whatever the number
-// of anchor pairs; the passes are chained as programmatic dependents (the transport releases
-// the blend at its end), the full-tile chain on the caller's stream and the edge-tile chain on
-// a second stream.  Global traffic beyond the algorithmic bytes: a second read of the anchors,
-// the records (120 floats per tile, pair and chunk) and, for bf16, the blend matrices (32 KB
-// per tile and target, read from L2 by every channel chunk).
+// of anchor pairs.  Global traffic beyond the algorithmic bytes: a second read of the anchors
+// (bf16: of each anchor once per pair and pass, from L2) and the records.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -157,8 +163,6 @@ struct ParKArgs {
   const float* wch;
   float* rec;     // workspace [tile][pair j][chunk][kRec]: each chunk's Z / W record
   float* trans;   // workspace [tile][pair j][2][kNB]: theta and g per bin
-  char* img;      // workspace [tile][target][kImgBytes]: blend matrices (bf16 runs), or null
-  int n_target;
   int F, Hg, Wg, C, n_chunk;             // n_chunk: channel chunks of kCC channels
   int tile_base;                         // global index of tile 0 of this launch's kind
   int th, tw, tiles_x, tiles_y, n_tile, n_tseg;
@@ -167,6 +171,16 @@ struct ParKArgs {
   int pair_tbeg[CAST_MAX_ANCHORS + 1];   // targets of pair j (anchors j-1, j) in [tbeg[j], tbeg[j+1])
   int target_frame[CAST_MAX_FRAMES];
   float target_alpha[CAST_MAX_FRAMES];
+  // bf16 path (tensor cores)
+  int n_full;                            // 8x8 tiles (tiles 0 .. n_full-1; the others follow)
+  int n_act, n_grp;                      // pairs with targets; groups of up to two targets of a pair
+  int st_parts, st_cpp, bl_parts, bl_cpp;   // channel-chunk ranges of K_stats_tc / K_blend_tc and chunks in each
+  // per tile shape (bit 0: last column of tiles, truncated; bit 1: last row): where the stored bin
+  // b's sums stand in a record (BinSlot), and the bin of each slot (255: none)
+  unsigned char bin_slot[4][40], slot_bin[4][34];
+  unsigned char act_pair[CAST_MAX_ANCHORS];
+  unsigned char grp_pair[CAST_MAX_FRAMES], grp_nt[CAST_MAX_FRAMES];
+  short grp_t0[CAST_MAX_FRAMES];
   int seg_pair0[CAST_MAX_ANCHORS];       // time segment s covers pairs seg_pair0[s] .. seg_pair1[s]
   int seg_pair1[CAST_MAX_ANCHORS];
   float tau_low, tau_high, q, T, eps, eta_rel, eta_abs, band;
@@ -176,13 +190,6 @@ struct ParKArgs {
   // 0 = not needed (Z at DC) or identically zero (Im Z at self-conjugate bins)
   signed char fast_src[kNV];
 };
-
-template <typename T>
-__device__ __forceinline__ float to_f32(T v);
-template <>
-__device__ __forceinline__ float to_f32<float>(float v) { return v; }
-template <>
-__device__ __forceinline__ float to_f32<__nv_bfloat16>(__nv_bfloat16 v) { return __bfloat162float(v); }
 
 
 struct TileGeom {
@@ -264,8 +271,7 @@ __device__ __forceinline__ void sincos_reduced(float x, float* s, float* c) {
 // whether the band cut forces g = 0.
 struct BinInfo {
   float tau[kNB], kap[kNB];
-  int rep[kNB];
-  unsigned char valid[kNB], selfc[kNB], mirror[kNB], cut[kNB];
+  unsigned char rep[kNB], valid[kNB], selfc[kNB], mirror[kNB], cut[kNB];
 };
 
 __device__ void bin_info(const ParKArgs& a, const TileGeom& g, BinInfo& bi, int tid) {
@@ -278,7 +284,7 @@ __device__ void bin_info(const ParKArgs& a, const TileGeom& g, BinInfo& bi, int 
   bi.valid[b] = valid;
   bi.selfc[b] = selfc;
   bi.mirror[b] = mirror;
-  bi.rep[b] = mirror ? (g.h - ky) * 5 + kx : b;
+  bi.rep[b] = (unsigned char)(mirror ? (g.h - ky) * 5 + kx : b);
   bi.kap[b] = (valid && b != 0) ? (edge ? 1.f : 2.f) : 0.f;
   const int kys = ky <= (g.h - 1) / 2 ? ky : ky - g.h;
   const float hh = (float)(g.h / 2) / (float)g.h, ww = (float)hw2 / (float)g.w;
@@ -367,127 +373,6 @@ __device__ void tile_transport(const ParKArgs& a, const TileGeom& g, const BinIn
   }
 }
 
-// ------------------------------------------------------------------ blend matrices
-constexpr int kImgTerm = 64 * 128 * 2;   // one bf16 piece of one target's [64][128] matrix, 16 KB
-constexpr int kImgBytes = 2 * kImgTerm;  // both pieces (hi, lo): 32 KB per (tile, target)
-
-// The blend matrices of the targets t_begin <= t < t_end of one (tile, pair), written as UMMA operand images
-// (K-major, 128-byte swizzle, K-blocks of 64 tokens 8 KB apart, two bf16 pieces kImgTerm apart):
-// row m = output token 8 yo + xo, column 64 side + 8 yi + xi = input token of anchor a (side 0)
-// or b (side 1); entry h_side((yo - yi) mod h, (xo - xi) mod w) with
-// h_side(d) = (1 / (h w)) sum over stored bins of kappa' Re(phi_side e^{2 pi i (ky dy / h + kx dx / w)}),
-// kappa' = 1 on the kx = 0 and Nyquist columns (every ky stored), 2 elsewhere;
-// phi_a = (1 - alpha) e^{i g alpha theta}, phi_b = alpha e^{-i g (1 - alpha) theta}.  128 threads.
-// FULL8: an 8x8 tile, where every twiddle is an 8th root of unity and every index a mask (the
-// same values, summed in the same order, as the general form).
-template <bool FULL8>
-__device__ void build_blend_images(const ParKArgs& a, const TileGeom& g, const BinInfo& bi,
-                                   const float* th, const float* gate, int tg, int t_begin, int t_end,
-                                   int tid) {
-  __shared__ float2 s_cs[64];
-  __shared__ unsigned char s_ym[8][8], s_xm[5][8];
-  __shared__ float4 s_phi[kNB];
-  __shared__ float s_h[2][64];
-  const int h = FULL8 ? 8 : g.h, w = FULL8 ? 8 : g.w, n = h * w;
-  if (FULL8) {
-    // e^{2 pi i q / 8} at s_cs[q]
-    if (tid < 8) {
-      float sv, cv;
-      sincospif((float)tid / 4.f, &sv, &cv);
-      s_cs[tid] = make_float2(cv, sv);
-    }
-  } else if (tid < 64) {
-    if (tid < n) {
-      float sv, cv;
-      sincospif(2.f * (float)tid / (float)n, &sv, &cv);
-      s_cs[tid] = make_float2(cv, sv);
-    }
-    s_ym[tid >> 3][tid & 7] = (unsigned char)(((tid >> 3) * (tid & 7)) % h);
-  } else if (tid < 64 + 40) {
-    const int e = tid - 64;
-    s_xm[e >> 3][e & 7] = (unsigned char)(((e >> 3) * (e & 7)) % w);
-  }
-  const float inv_n = 1.f / (float)n;
-  const int side = tid >> 6, d = tid & 63, dy0 = d >> 3, dx0 = d & 7;
-  for (int t = t_begin; t < t_end; ++t) {
-    const float al = a.target_alpha[t];
-    if (tid < kNB) {
-      const int b = tid, kx = b % 5;
-      float4 ph = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (bi.valid[b]) {
-        const bool edge = kx == 0 || ((w % 2 == 0) && kx == w / 2);
-        const float kap = (edge ? 1.f : 2.f) * inv_n;
-        float sa, ca, sb, cb;
-        const float gt = gate[b] * th[b];
-        sincosf(gt * al, &sa, &ca);
-        sincosf(-gt * (1.f - al), &sb, &cb);
-        ph = make_float4(kap * (1.f - al) * ca, kap * (1.f - al) * sa, kap * al * cb, kap * al * sb);
-      }
-      s_phi[b] = ph;
-    }
-    __syncthreads();
-    if (FULL8) {
-      float acc = 0.f;
-#pragma unroll
-      for (int ky = 0; ky < 8; ++ky) {
-        const int ry = ky * dy0;
-#pragma unroll
-        for (int kx = 0; kx < 5; ++kx) {
-          const float2 e = s_cs[(ry + kx * dx0) & 7];
-          const float4 ph = s_phi[ky * 5 + kx];
-          const float pr = side ? ph.z : ph.x, pi = side ? ph.w : ph.y;
-          acc = fmaf(pr, e.x, fmaf(-pi, e.y, acc));
-        }
-      }
-      s_h[side][d] = acc;
-    } else {
-      float acc = 0.f;
-      if (dy0 < h && dx0 < w) {
-        for (int b = 0; b < kNB; ++b) {
-          const int ky = b / 5, kx = b % 5;
-          if (ky >= h || kx > w / 2) continue;
-          int p = (int)s_ym[ky][dy0] * w + (int)s_xm[kx][dx0] * h;
-          if (p >= n) p -= n;
-          const float2 e = s_cs[p];
-          const float4 ph = s_phi[b];
-          const float pr = side ? ph.z : ph.x, pi = side ? ph.w : ph.y;
-          acc = fmaf(pr, e.x, fmaf(-pi, e.y, acc));
-        }
-      }
-      s_h[side][d] = acc;
-    }
-    __syncthreads();
-    // 16-byte chunk q = 128 it + tid of a piece: side q >> 9, output token (row) m = (q >> 3) & 63,
-    // stored chunk q & 7 = input row yi ^ (m & 7); a warp writes 512 contiguous bytes per piece
-    uint8_t* img = reinterpret_cast<uint8_t*>(a.img) + ((int64_t)tg * a.n_target + t) * kImgBytes;
-#pragma unroll
-    for (int it = 0; it < 8; ++it) {
-      const int q = it * 128 + tid, sd = q >> 9, m = (q >> 3) & 63, yi = (q & 7) ^ (m & 7);
-      const int yo = m >> 3, xo = m & 7;
-      const bool row_ok = FULL8 || (yo < h && xo < w && yi < h);
-      const int dy = FULL8 ? (yo - yi) & 7 : yo - yi + (yo < yi ? h : 0);
-      float v[8];
-#pragma unroll
-      for (int xi = 0; xi < 8; ++xi) {
-        const int dx = FULL8 ? (xo - xi) & 7 : xo - xi + (xo < xi ? w : 0);
-        v[xi] = (FULL8 || (row_ok && xi < w)) ? s_h[sd][dy * 8 + dx] : 0.f;
-      }
-      uint32_t hi[4], lo[4];
-#pragma unroll
-      for (int u = 0; u < 8; u += 2) {
-        const __nv_bfloat162 b1 = __floats2bfloat162_rn(v[u], v[u + 1]);
-        const __nv_bfloat162 b2 = __floats2bfloat162_rn(v[u] - __low2float(b1), v[u + 1] - __high2float(b1));
-        hi[u / 2] = *reinterpret_cast<const uint32_t*>(&b1);
-        lo[u / 2] = *reinterpret_cast<const uint32_t*>(&b2);
-      }
-      const int off = q << 4;   // side * 8192 + m * 128 + ((yi ^ (m & 7)) << 4)
-      *reinterpret_cast<uint4*>(img + off) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
-      *reinterpret_cast<uint4*>(img + kImgTerm + off) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
-    }
-    __syncthreads();   // s_phi and s_h are rewritten for the next target
-  }
-}
-
 __device__ __forceinline__ void grid_dependency_wait() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }
@@ -495,23 +380,17 @@ __device__ __forceinline__ void launch_dependents() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
-// Dynamic shared memory of a streaming CTA with cc channels: a ring of n_stages<T> TMA stages
-// (one anchor tile each, 128-byte aligned; two for bf16, one for f32 so that three CTAs still
-// fit an SM) and the previous anchor's spectrum [value][thread].
-template <typename T>
-__host__ __device__ constexpr int n_stages() { return sizeof(T) == 2 ? 2 : 1; }
-template <typename T>
-__host__ __device__ constexpr size_t stage_bytes(int cc) { return (size_t)64 * cc * sizeof(T); }
+// Dynamic shared memory of a streaming f32 CTA with cc channels: the TMA stage (one anchor tile,
+// 128-byte aligned; one, so that three CTAs fit an SM) and the previous anchor's spectrum
+// [value][thread].
+__host__ __device__ constexpr size_t stage_bytes(int cc) { return (size_t)64 * cc * sizeof(float); }
 __host__ __device__ constexpr size_t spec_bytes(int cc) { return (size_t)2 * kNB * cc * sizeof(float); }
-template <typename T>
-__host__ __device__ constexpr size_t par_dyn_smem(int cc) {
-  return n_stages<T>() * stage_bytes<T>(cc) + spec_bytes(cc) + 128;
-}
+__host__ __device__ constexpr size_t par_dyn_smem(int cc) { return stage_bytes(cc) + spec_bytes(cc) + 128; }
 
 // K_stats (STATS) and K_blend (!STATS): grid (n_chunk, n_tiles_of_kind * n_tseg), CC threads,
 // one channel each.  A time segment covers the anchor pairs seg_pair0 .. seg_pair1 (it starts
 // one anchor earlier).  FULL: every tile of the launch is 8x8 (the specialised fast path).
-template <typename T, int CC, bool FULL, bool STATS>
+template <int CC, bool FULL, bool STATS>
 __global__ void __launch_bounds__(CC, 3)
     k_par(const __grid_constant__ CUtensorMap tm, const __grid_constant__ ParKArgs a) {
   extern __shared__ uint8_t dsm_raw[];
@@ -519,12 +398,11 @@ __global__ void __launch_bounds__(CC, 3)
   uint8_t* dsm = dsm_raw + (((raw + 127u) & ~127u) - raw);   // TMA boxes without swizzle: 128 B
   constexpr int cc = CC;
   constexpr int nwarp = CC / 32;
-  constexpr int kStages = n_stages<T>();
-  T* stages = reinterpret_cast<T*>(dsm);       // kStages x [y][x][channel] of one anchor tile
-  float* s_fprev = reinterpret_cast<float*>(dsm + kStages * stage_bytes<T>(cc));   // [value][thread]
+  float* stage = reinterpret_cast<float*>(dsm);                      // [y][x][channel] of one anchor tile
+  float* s_fprev = reinterpret_cast<float*>(dsm + stage_bytes(cc));   // [value][thread]
   __shared__ float s_red[STATS ? nwarp : 1][128];
   __shared__ float4 s_coef[STATS ? 1 : kCoefBatch][kNB];
-  __shared__ __align__(8) uint64_t s_full[kStages];
+  __shared__ __align__(8) uint64_t s_full;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int chunk = blockIdx.x;
   const int tile = blockIdx.y / a.n_tseg, seg = blockIdx.y - tile * a.n_tseg;
@@ -535,17 +413,13 @@ __global__ void __launch_bounds__(CC, 3)
   const bool active = c < a.C;
   const float wc = active ? (a.wch ? __ldg(a.wch + c) : 1.f) : 0.f;
   // bytes one TMA box delivers: cc channels x tile_w x tile_h (must match the tensor map)
-  const uint32_t box_bytes = (uint32_t)(cc * a.tw * a.th * sizeof(T));
+  const uint32_t box_bytes = (uint32_t)(cc * a.tw * a.th * sizeof(float));
   if (tid == 0) {
-    for (int st = 0; st < kStages; ++st) mbar_init(&s_full[st], 1);
+    mbar_init(&s_full, 1);
     fence_barrier_init();
     tma_prefetch_desc(&tm);
-    // the first kStages anchors of the segment are in flight at once
-    for (int st = 0; st < kStages && j0 + st <= j1; ++st) {
-      mbar_arrive_expect_tx(&s_full[st], box_bytes);
-      tma_load_4d(stages + st * (stage_bytes<T>(cc) / sizeof(T)), &tm, &s_full[st], chunk * cc, g.x0,
-                  g.y0, a.anchor_frame[j0 + st]);
-    }
+    mbar_arrive_expect_tx(&s_full, box_bytes);
+    tma_load_4d(stage, &tm, &s_full, chunk * cc, g.x0, g.y0, a.anchor_frame[j0]);
   }
   launch_dependents();
   __syncthreads();
@@ -553,36 +427,33 @@ __global__ void __launch_bounds__(CC, 3)
   if (!STATS) grid_dependency_wait();
   bool ok = true;          // CTA-uniform; after a failed wait no more TMA is issued
   const int64_t frame_elems = (int64_t)a.Hg * a.Wg * a.C;
-  T* out = reinterpret_cast<T*>(a.r);
+  float* out = reinterpret_cast<float*>(a.r);
 
   for (int j = j0; j <= j1; ++j) {
     float re[8][5], im[8][5];
     {
-      const int it = j - j0, st = it % kStages;
-      const T* stage = stages + st * (stage_bytes<T>(cc) / sizeof(T));
-      const bool got = ok && mbar_wait(&s_full[st], (uint32_t)(it / kStages) & 1u, a.wait_ns);
+      const bool got = ok && mbar_wait(&s_full, (uint32_t)(j - j0) & 1u, a.wait_ns);
       float x[8][8];
       if (FULL) {
 #pragma unroll
         for (int y = 0; y < 8; ++y)
 #pragma unroll
-          for (int xx = 0; xx < 8; ++xx) x[y][xx] = to_f32(stage[(y * 8 + xx) * cc + tid]);
+          for (int xx = 0; xx < 8; ++xx) x[y][xx] = stage[(y * 8 + xx) * cc + tid];
       } else {
 #pragma unroll
         for (int y = 0; y < 8; ++y)
 #pragma unroll
           for (int xx = 0; xx < 8; ++xx)
-            x[y][xx] = (y < g.h && xx < g.w) ? to_f32(stage[(y * a.tw + xx) * cc + tid]) : 0.f;
+            x[y][xx] = (y < g.h && xx < g.w) ? stage[(y * a.tw + xx) * cc + tid] : 0.f;
       }
-      // the stage is free: the anchor kStages ahead goes into it while this one is transformed
+      // the stage is free: the next anchor goes into it while this one is transformed
       if (__syncthreads_or(ok && !got)) {
         if (tid == 0) atomicExch(&g_par_error, 1u);
         ok = false;
       }
-      if (ok && tid == 0 && j + kStages <= j1) {
-        mbar_arrive_expect_tx(&s_full[st], box_bytes);
-        tma_load_4d(const_cast<T*>(stage), &tm, &s_full[st], chunk * cc, g.x0, g.y0,
-                    a.anchor_frame[j + kStages]);
+      if (ok && tid == 0 && j < j1) {
+        mbar_arrive_expect_tx(&s_full, box_bytes);
+        tma_load_4d(stage, &tm, &s_full, chunk * cc, g.x0, g.y0, a.anchor_frame[j + 1]);
       }
       if (FULL) dft::fwd2d(x, 8, 8, re, im);
       else dft::fwd2d(x, g.h, g.w, re, im);
@@ -672,7 +543,7 @@ __global__ void __launch_bounds__(CC, 3)
             hr[ky][kx] = cf.x * ar - cf.y * ai + cf.z * br - cf.w * bi;
             hi[ky][kx] = cf.x * ai + cf.y * ar + cf.z * bi + cf.w * br;
           }
-          T* dst = out + (int64_t)a.target_frame[t0 + k] * frame_elems +
+          float* dst = out + (int64_t)a.target_frame[t0 + k] * frame_elems +
                    ((int64_t)g.y0 * a.Wg + g.x0) * a.C + c;
           const int64_t row_step = (int64_t)a.Wg * a.C;
           const int w = FULL ? 8 : g.w, C = a.C;
@@ -680,10 +551,10 @@ __global__ void __launch_bounds__(CC, 3)
           asm volatile("" ::: "memory");
           auto emit = [&](int yy, const float* row) {
             if (!active) return;
-            T* d = dst + yy * row_step;
+            float* d = dst + yy * row_step;
 #pragma unroll
             for (int xx = 0; xx < 8; ++xx)
-              if (xx < w) d[(int64_t)xx * C] = T(row[xx]);
+              if (xx < w) d[(int64_t)xx * C] = row[xx];
           };
           if (FULL) dft::inv2d_emit(hr, hi, 8, 8, emit);
           else dft::inv2d_emit(hr, hi, g.h, g.w, emit);
@@ -702,19 +573,417 @@ __global__ void __launch_bounds__(CC, 3)
   }
 }
 
-// K_transport: grid (n_tiles_of_kind, n_anchor - 1, z), 128 threads; block y = pair j - 1.  With
-// blend matrices (bf16) block z builds the matrix of the pair's target z (z < the largest target
-// count of a pair; every block of a (tile, pair) solves the same transport), else z = 0 only.
+// ------------------------------------------------------------------ K_stats_tc (bf16)
+// Z and W of every anchor pair with targets on the tensor cores.  A unit is one (tile, pair) with
+// a range of 128-channel chunks.  Per chunk the two anchors' tiles arrive by TMA ([8 x 8 tokens]
+// [channels], 128-byte swizzle) and one UMMA chain each transforms them: D[channel][column] =
+// X^T F with the tile's DFT as a 112-column operand in shared memory, M = 128 channels, K = 64
+// tokens, D in TMEM.  A thread then owns one channel: it reads both spectra from TMEM and adds
+// its products to 98 registers (Re Z, Im Z, W of 30 complex bins, Z and W of 4 real ones), which
+// are reduced over the channels once per unit.
+// The 8x8 transform is exact: every twiddle is an integer plus an integer times sqrt(1/2), so the
+// columns hold the two integer parts (0, +-1) of each value and the thread forms A + sqrt(1/2) B
+// in f32.  Other tile shapes hold the twiddles in three bf16 pieces (24 bits), accumulated into
+// the A columns.
+// Bound by issue slots: 16 warps of ~250 instructions per chunk (130 of them FMAs of the 8 bins of
+// a warpgroup), ~1,100 cycles a chunk.  The register transform it replaces spent 1,400
+// instructions per channel and anchor, half of them on transposing every chunk's sums between
+// lanes: 45 us for the 50 full tiles and 22 us beside it for the 10 edge tiles of the
+// HY-World-shaped call; this kernel takes 42 us for both.
+constexpr int kStSumWarps = 16, kStSumThreads = 32 * kStSumWarps;
+constexpr int kStThreads = 128 + kStSumThreads, kStStages = 4;
+constexpr int kNCpx = 30, kNOdd = 24, kNReal = 4;       // complex bins (the first 24 with sqrt(1/2) parts), real bins
+constexpr int kStN = 112;                               // columns: four warpgroups of 28
+constexpr int kStTile = 64 * 128 * 2;                   // one anchor tile, 16 KB
+constexpr int kStPiece = kStN * 128;                    // one operand piece [112][64] bf16, 14 KB
+constexpr int kStSums = 3 * kNCpx + 2 * kNReal;         // 98
+constexpr int kQOdd = kNOdd / 4, kQCpx = kQOdd + 2;     // complex bins of a warpgroup: six odd ones and a pair of even
+constexpr int kQCols = kStN / 4;                        // its columns: A and B (re, im) of the odd bins, then the pair or the reals
+constexpr int kStSmem = kStStages * 2 * kStTile + 3 * kStPiece + 2 * kStSumWarps * 32 * 4 + 1024;
+static_assert(kStSums <= kRec, "record slots");
+
+// Record slots of the stored bins of an h x w tile: complex representatives in bin order (8x8:
+// those with an odd frequency first), self-conjugate (real) bins 0..3 apart; mirrors point at
+// their representative.  255: not stored.
+constexpr int kSlotMirror = 64, kSlotReal = 128;
+void make_slots(int h, int w, unsigned char* bin_slot, unsigned char* slot_bin) {
+  const bool full = h == 8 && w == 8;
+  for (int q = 0; q < kNCpx + kNReal; ++q) slot_bin[q] = 255;
+  int n_cpx = 0, n_even = kNOdd, n_real = 0;
+  for (int pass = 0; pass < 2; ++pass)   // representatives, then mirrors
+    for (int b = 0; b < kNB; ++b) {
+      const int ky = b / 5, kx = b % 5;
+      const bool edge = kx == 0 || (w % 2 == 0 && kx == w / 2);
+      const bool real = edge && (ky == 0 || (h % 2 == 0 && 2 * ky == h));
+      const bool mirror = edge && !real && 2 * ky > h;
+      if (ky >= h || kx > w / 2) {
+        bin_slot[b] = 255;
+      } else if (mirror) {
+        if (pass == 1) bin_slot[b] = bin_slot[(h - ky) * 5 + kx] | kSlotMirror;
+      } else if (pass == 0) {
+        const int slot = real ? n_real++ : full && ((ky | kx) & 1) == 0 ? n_even++ : n_cpx++;
+        bin_slot[b] = (unsigned char)(slot | (real ? kSlotReal : 0));
+        slot_bin[real ? kNCpx + slot : slot] = (unsigned char)b;
+      }
+    }
+}
+
+__device__ __forceinline__ int tile_shape(const ParKArgs& a, const TileGeom& g) {
+  return (g.h < a.th ? 2 : 0) + (g.w < a.tw ? 1 : 0);
+}
+
+__device__ __forceinline__ void stats_sync() { asm volatile("bar.sync 2, %0;" ::"n"(kStSumThreads) : "memory"); }
+
+// A tile's transform as the swizzled K-major operand [112 columns][64 tokens] (one piece for
+// 8x8, three for other shapes).  Runs once or twice per CTA, when its instructions are not yet
+// cached, so the code is kept short (unrolled, it took 6 us of the kernel).
+__device__ void build_dft_operand(const ParKArgs& a, const TileGeom& g, uint8_t* img, int tid) {
+  // rows 0-2: bf16 pieces of cos and -sin of m / turn of a turn; 8x8: row 0 the integers, row 1
+  // the factors of sqrt(1/2)
+  __shared__ unsigned short s_tab[3][2][64];
+  __shared__ unsigned char bins[kNCpx + kNReal];
+  const int h = g.h, w = g.w;
+  const bool full = h == 8 && w == 8;
+  const int turn = full ? 8 : h * w;
+  if (tid < 2 * 64 && (tid & 63) < turn) {
+    const int im = tid >> 6, m = tid & 63;
+    float sv, cv;
+    sincospif(2.f * (float)m / (float)turn, &sv, &cv);
+    float v = im ? -sv : cv;
+    const bool odd = full && (m & 1);
+    if (full) v = odd ? copysignf(1.f, v) : rintf(v);
+#pragma unroll 1
+    for (int p = 0; p < 3; ++p) {
+      const __nv_bfloat16 b = __float2bfloat16_rn(full ? (p == (odd ? 1 : 0) ? v : 0.f) : v);
+      s_tab[p][im][m] = __bfloat16_as_ushort(b);
+      if (!full) v -= __bfloat162float(b);
+    }
+  } else if (tid >= 128 && tid < 128 + kNCpx + kNReal) {
+    bins[tid - 128] = a.slot_bin[tile_shape(a, g)][tid - 128];
+  }
+  stats_sync();
+#pragma unroll 1
+  for (int e = tid; e < kStN * 8; e += kStSumThreads) {
+    const int col = e >> 3, y = e & 7;
+    const int wg = col / kQCols, r = col - wg * kQCols;
+    const bool bpart = r >= 2 * kQOdd && r < 4 * kQOdd;
+    int slot = wg * kQOdd + (r % (2 * kQOdd)) / 2, im = r & 1;
+    if (r >= 4 * kQOdd && wg < 3) slot = kNOdd + 2 * wg + (r - 4 * kQOdd) / 2;
+    else if (r >= 4 * kQOdd) slot = kNCpx + r - 4 * kQOdd, im = 0;
+    const int b = bins[slot], ky = b / 5, kx = b % 5;
+    const bool live = b != 255 && y < h && (full || !bpart);
+    uint8_t* dst = img + col * 128 + ((y ^ (col & 7)) << 4);
+#pragma unroll 1
+    for (int p = 0; p < (full ? 1 : 3); ++p) {
+      // e^{-2 pi i (ky y / h + kx x / w)}: angle m in units of 1 / turn, stepping with x
+      const unsigned short* t = s_tab[full ? (int)bpart : p][im];
+      const int dm = full ? kx : (kx * h) % turn;
+      int m = (full ? ky * y : ky * y * w) % turn;
+#pragma unroll 1
+      for (int x = 0; x < 8; ++x) {
+        *reinterpret_cast<unsigned short*>(dst + p * kStPiece + 2 * x) = live && x < w ? t[m] : (unsigned short)0;
+        m += dm;
+        if (m >= turn) m -= turn;
+      }
+    }
+  }
+}
+
+// One anchor's tile of 128 channels into [64-channel half][8 y + x] of shared memory.  Tiles of
+// other sides than 8x8 are loaded row by row, so that no token of a neighbouring tile is read; the
+// other tokens of their stages are zero (zero_stages, once per CTA) and stay so.
+__device__ __forceinline__ bool whole_tiles(const ParKArgs& a) { return a.th == 8 && a.tw == 8; }
+__device__ __forceinline__ uint32_t anchor_tile_bytes(const ParKArgs& a) { return (uint32_t)(2 * a.th * a.tw * 128); }
+__device__ __forceinline__ void load_anchor_tile(const ParKArgs& a, const CUtensorMap* tm, uint8_t* dst, uint64_t* bar,
+                                                 int ch, const TileGeom& g, int frame) {
+  for (int b = 0; b < 2; ++b) {
+    if (whole_tiles(a)) {
+      tma_load_4d(dst + b * 8192, tm, bar, ch + b * 64, g.x0, g.y0, frame);
+    } else {
+      for (int y = 0; y < a.th; ++y)
+        tma_load_4d(dst + b * 8192 + y * 1024, tm, bar, ch + b * 64, g.x0, g.y0 + y, frame);
+    }
+  }
+}
+__device__ __forceinline__ void zero_stages(const ParKArgs& a, uint8_t* p, int bytes) {
+  if (whole_tiles(a)) return;
+  for (int e = threadIdx.x * 16; e < bytes; e += blockDim.x * 16) *reinterpret_cast<uint4*>(p + e) = make_uint4(0u, 0u, 0u, 0u);
+  fence_proxy_async_smem();
+}
+
+__device__ __forceinline__ TileGeom any_tile(const ParKArgs& a, int tile) {
+  return tile < a.n_full ? tile_geom(a, tile, true) : tile_geom(a, tile - a.n_full, false);
+}
+
+template <bool WEIGHTED>
+__global__ void __launch_bounds__(kStThreads, 1)
+    k_par_stats_tc(const __grid_constant__ CUtensorMap tm, const __grid_constant__ ParKArgs a) {
+  extern __shared__ uint8_t dsm_raw[];
+  const uint32_t raw_addr = smem_u32(dsm_raw);
+  uint8_t* dsm = dsm_raw + (((raw_addr + 1023u) & ~1023u) - raw_addr);
+  uint8_t* s_x = dsm;
+  uint8_t* s_img = dsm + kStStages * 2 * kStTile;
+  float* s_red = reinterpret_cast<float*>(s_img + 3 * kStPiece);   // [2][16 warps][32]
+  __shared__ __align__(8) uint64_t b_full[kStStages], b_empty[kStStages], b_dfull[2], b_dempty[2], b_img;
+  __shared__ uint32_t s_tmem;
+  __shared__ volatile int s_abort;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int nck = a.n_chunk, n_units = a.n_tile * a.n_act * a.st_parts;
+  const uint64_t lim = a.wait_ns;
+  auto wait = [&](uint64_t* bar, uint32_t parity) -> bool {
+    if (mbar_try_wait(bar, parity)) return true;
+    if (s_abort) return false;
+    if (mbar_wait(bar, parity, lim)) return true;
+    s_abort = 1;
+    atomicExch(&g_par_error, 1u);
+    return false;
+  };
+  if (tid == 0) {
+    for (int s = 0; s < kStStages; ++s) {
+      mbar_init(&b_full[s], 1);
+      mbar_init(&b_empty[s], 1);
+    }
+    for (int b = 0; b < 2; ++b) {
+      mbar_init(&b_dfull[b], 1);
+      mbar_init(&b_dempty[b], kStSumWarps);
+    }
+    mbar_init(&b_img, 1);
+    fence_barrier_init();
+    s_abort = 0;
+  }
+  if (warp == 1) {
+    tmem_alloc(&s_tmem, 512);
+    tmem_relinquish();
+    tc_fence_before();
+  }
+  zero_stages(a, s_x, kStStages * 2 * kStTile);
+  launch_dependents();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = s_tmem;
+  // unit u -> (tile, pair, chunk range): pairs innermost, so that a tile's anchors are read
+  // from L2 by the CTAs of neighbouring units
+  struct Unit {
+    int tile, j, part, c0, c1;
+  };
+  auto unit_of = [&](int u) {
+    Unit x;
+    const int per = a.n_act * a.st_parts;
+    x.tile = u / per;
+    const int r = u - x.tile * per;
+    x.part = r / a.n_act;
+    x.j = a.act_pair[r - x.part * a.n_act];
+    x.c0 = x.part * a.st_cpp;
+    x.c1 = min(nck, x.c0 + a.st_cpp);
+    return x;
+  };
+
+  if (warp < 4) {
+    if (warp == 0 && lane == 0) {
+      // -------------------------------------------------------------- anchor producer
+      tma_prefetch_desc(&tm);
+      int n = 0;
+      bool ok = true;
+      for (int u = blockIdx.x; ok && u < n_units; u += gridDim.x) {
+        const Unit x = unit_of(u);
+        const TileGeom g = any_tile(a, x.tile);
+        for (int c = x.c0; c < x.c1; ++c, ++n) {
+          const int s = n % kStStages;
+          if (n >= kStStages && !wait(&b_empty[s], (uint32_t)((n / kStStages) - 1) & 1u)) { ok = false; break; }
+          mbar_arrive_expect_tx(&b_full[s], 2 * anchor_tile_bytes(a));
+          for (int q = 0; q < 2; ++q)
+            load_anchor_tile(a, &tm, s_x + (2 * s + q) * kStTile, &b_full[s], c * 128, g, a.anchor_frame[x.j - 1 + q]);
+        }
+      }
+      if (!ok)   // the copies still in flight land before the shared memory is released
+        for (int l = n > kStStages ? n - kStStages : 0; l < n; ++l)
+          mbar_wait(&b_full[l % kStStages], (uint32_t)(l / kStStages) & 1u, lim);
+    } else if (warp & 1) {
+      // -------------------------------------------------------------- UMMA issuers (converged)
+      // warps 1 and 3 take alternate chunks and accumulators: the ~500 cycles that an issuer
+      // spends on waits and commits per chunk pass while the other one's UMMAs run
+      constexpr uint32_t idesc = idesc_bf16_f32(128, kStN, true, false);
+      const int buf = warp >> 1;
+      const uint32_t tmu = __shfl_sync(0xffffffffu, tmem, 0) + (uint32_t)(buf * 256);
+      const uint32_t xb = __shfl_sync(0xffffffffu, smem_u32(s_x), 0), ib = __shfl_sync(0xffffffffu, smem_u32(s_img), 0);
+      const uint64_t dx = sdesc_sw128(xb, 8192, 1024), di = sdesc_sw128(ib, 16, 1024);
+      const bool lead = elect_one();
+      int n = 0, last = -1, shape = -1, builds = 0;
+      bool ok = true;
+      for (int u = blockIdx.x; ok && u < n_units; u += gridDim.x) {
+        const Unit x = unit_of(u);
+        const TileGeom g = any_tile(a, x.tile);
+        if (g.h * 16 + g.w != shape) {
+          shape = g.h * 16 + g.w;
+          if (!(ok = __all_sync(0xffffffffu, wait(&b_img, (uint32_t)builds++ & 1u)))) break;
+        }
+        const bool pieces = !(g.h == 8 && g.w == 8);
+        for (int c = x.c0; c < x.c1; ++c, ++n) {
+          if ((n & 1) != buf) continue;
+          const int s = n % kStStages;
+          // half of the warp waits for the anchors, half for the accumulator
+          const bool w = lane < 16 ? wait(&b_full[s], (uint32_t)(n / kStStages) & 1u)
+                                   : n < 2 || wait(&b_dempty[buf], (uint32_t)((n >> 1) - 1) & 1u);
+          if (!(ok = __all_sync(0xffffffffu, w))) break;
+          tc_fence_after();
+          if (lead) {
+            const uint64_t da = dx + (uint64_t)(2 * s * (kStTile >> 4));
+            auto chain = [&](int q, int p) {
+#pragma unroll
+              for (int kk = 0; kk < 4; ++kk)
+                umma_bf16_ss(tmu + (uint32_t)(q * 128), da + (uint64_t)(q * (kStTile >> 4) + kk * (2048 >> 4)),
+                             di + (uint64_t)(p * (kStPiece >> 4) + kk * 2), idesc, (p | kk) ? 1u : 0u);
+            };
+            chain(0, 0);
+            if (pieces) chain(0, 1), chain(0, 2);
+            chain(1, 0);
+            if (pieces) chain(1, 1), chain(1, 2);
+            umma_commit(&b_empty[s]);
+            umma_commit(&b_dfull[buf]);
+          }
+          __syncwarp();
+          last = n;
+        }
+      }
+      // the UMMAs issued so far have completed before shared memory and TMEM are released
+      if (last >= 0) mbar_wait(&b_dfull[buf], (uint32_t)(last >> 1) & 1u, lim);
+      __syncwarp();
+    }
+  } else {
+    // ---------------------------------------------------------------- sums
+    // One channel per thread (and per TMEM lane) in each of four warpgroups, a quarter of the bins
+    // in each: four warps per scheduler cover the latency of the TMEM reads and square roots
+    // (two warpgroups with half of the bins took 1,160 cycles a chunk).  Warpgroup w has the
+    // complex bins 6 w .. 6 w + 5 and 24 + 2 w, 25 + 2 w, the last one the real bins instead.
+    const int wg = (warp >> 2) - 1, q4 = warp & 3, ctid = tid - 128;
+    const uint32_t td0 = tmem + ((uint32_t)(q4 * 32) << 16);
+    constexpr float kR = 0.70710678118654752f;
+    int n = 0, shape = -1, flip = 0;
+    bool ok = true;
+    for (int u = blockIdx.x; u < n_units; u += gridDim.x, flip ^= 1) {
+      const Unit x = unit_of(u);
+      const TileGeom g = any_tile(a, x.tile);
+      if (g.h * 16 + g.w != shape) {
+        // every UMMA that read the operand has completed: its chunk has been waited for
+        shape = g.h * 16 + g.w;
+        build_dft_operand(a, g, s_img, ctid);
+        fence_proxy_async_smem();
+        stats_sync();
+        if (ctid == 0) mbar_arrive(&b_img);
+      }
+      // Re Z, Im Z, W of the complex bins; of the last warpgroup, Z of the real bins in zr[6],
+      // zr[7], zi[6], zi[7] and W in wv[6], wv[7], ex[0], ex[1]
+      float zr[kQCpx], zi[kQCpx], wv[kQCpx], ex[2] = {0.f, 0.f};
+#pragma unroll
+      for (int c = 0; c < kQCpx; ++c) zr[c] = zi[c] = wv[c] = 0.f;
+      // one complex bin; the weight goes on anchor a (w >= 0, so |w F_a| = w |F_a|)
+      float wc = 1.f;
+      auto add = [&](int s, float ra, float ia, float rb, float ib) {
+        if (WEIGHTED) {
+          ra *= wc;
+          ia *= wc;
+        }
+        zr[s] = fmaf(rb, ra, fmaf(ib, ia, zr[s]));
+        zi[s] = fmaf(ib, ra, fmaf(-rb, ia, zi[s]));
+        wv[s] += sqrt_approx(fmaf(ra, ra, ia * ia) * fmaf(rb, rb, ib * ib));
+      };
+      for (int c = x.c0; c < x.c1; ++c, ++n) {
+        const int buf = n & 1, ch = c * 128 + q4 * 32 + lane;
+        if (WEIGHTED) wc = ch < a.C ? __ldg(a.wch + ch) : 1.f;
+        if (!(ok = __all_sync(0xffffffffu, wait(&b_dfull[buf], (uint32_t)(n >> 1) & 1u)))) break;
+        tc_fence_after();
+        // the warpgroup's columns of anchors a and b, then the buffer goes back to its issuer
+        uint32_t va[64];
+        tmem_ld_x32_async(td0 + (uint32_t)(buf * 256 + wg * kQCols), va);
+        tmem_ld_x32_async(td0 + (uint32_t)(buf * 256 + 128 + wg * kQCols), va + 32);
+        tmem_wait_ld_x64(va);
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&b_dempty[buf]);
+        const float *fa = reinterpret_cast<const float*>(va), *fb = fa + 32;
+#pragma unroll
+        for (int e = 0; e < 2 * kQOdd; e += 2)   // A + sqrt(1/2) B
+          add(e / 2, fmaf(kR, fa[2 * kQOdd + e], fa[e]), fmaf(kR, fa[2 * kQOdd + e + 1], fa[e + 1]),
+              fmaf(kR, fb[2 * kQOdd + e], fb[e]), fmaf(kR, fb[2 * kQOdd + e + 1], fb[e + 1]));
+        fa += 4 * kQOdd;
+        fb += 4 * kQOdd;
+        if (wg < 3) {
+          add(kQOdd, fa[0], fa[1], fb[0], fb[1]);
+          add(kQOdd + 1, fa[2], fa[3], fb[2], fb[3]);
+        } else {
+          const float z0 = wc * fa[0] * fb[0], z1 = wc * fa[1] * fb[1], z2 = wc * fa[2] * fb[2], z3 = wc * fa[3] * fb[3];
+          zr[kQOdd] += z0;
+          zr[kQOdd + 1] += z1;
+          zi[kQOdd] += z2;
+          zi[kQOdd + 1] += z3;
+          wv[kQOdd] += fabsf(z0);
+          wv[kQOdd + 1] += fabsf(z1);
+          ex[0] += fabsf(z2);
+          ex[1] += fabsf(z3);
+        }
+      }
+      // sums over the channels by a warp transpose (8 Re Z | 8 Im Z | 8 W | 2 more), then over the
+      // warpgroup's four warps in order
+      {
+        float t[32];
+#pragma unroll
+        for (int e = 0; e < 32; ++e)
+          t[e] = e < kQCpx ? zr[e < kQCpx ? e : 0]
+               : e < 2 * kQCpx ? zi[e < 2 * kQCpx ? e - kQCpx : 0]
+               : e < 3 * kQCpx ? wv[e < 3 * kQCpx ? e - 2 * kQCpx : 0]
+               : e < 3 * kQCpx + 2 ? ex[e < 3 * kQCpx + 2 ? e - 3 * kQCpx : 0] : 0.f;
+        s_red[(flip * kStSumWarps + warp - 4) * 32 + lane] = warp_transpose_sum(t, lane);
+      }
+      // (the warps leave together: a thread left behind would wait in this barrier)
+      if (bar_sync_or(2, kStSumThreads, !ok || s_abort)) break;
+      if (ctid < kStSums) {
+        // record slot (30 Re Z | 30 Im Z | 30 W | 4 Z | 4 W) -> warpgroup and place in its sums
+        const int part = ctid / kNCpx, slot = ctid - part * kNCpx;
+        int of = 3, at;
+        if (part < 3) {
+          of = slot < kNOdd ? slot / kQOdd : (slot - kNOdd) >> 1;
+          at = part * kQCpx + (slot < kNOdd ? slot - of * kQOdd : kQOdd + ((slot - kNOdd) & 1));
+        } else {
+          const int r = slot & 3;   // Z: zr, zr, zi, zi; W: wv, wv, ex, ex
+          at = (slot < kNReal ? (r >> 1) : 2 + (r >> 1)) * kQCpx + (slot >= kNReal && r >= 2 ? 0 : kQOdd) + (r & 1);
+        }
+        float sum = 0.f;
+#pragma unroll
+        for (int w4 = 0; w4 < 4; ++w4) sum += s_red[(flip * kStSumWarps + of * 4 + w4) * 32 + at];
+        a.rec[(((int64_t)x.tile * a.n_anchor + x.j) * a.n_chunk + x.part) * kRec + ctid] = sum;
+      }
+      // the other half of s_red is written next, this one only after the next unit's barrier
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 1) tmem_dealloc(tmem, 512);
+}
+
+// Sum of `n` record entries kRec apart, in order, twelve loads in flight per round.
+__device__ __forceinline__ float record_sum(const float* r, int n) {
+  float sum = 0.f;
+  for (int q0 = 0; q0 < n; q0 += 12) {
+    float v[12];
+#pragma unroll
+    for (int u = 0; u < 12; ++u) v[u] = q0 + u < n ? __ldcg(r + (int64_t)(q0 + u) * kRec) : 0.f;
+#pragma unroll
+    for (int u = 0; u < 12; ++u) sum += v[u];
+  }
+  return sum;
+}
+
+// ------------------------------------------------------------------ K_transport (f32)
+// grid (n_tiles_of_kind, n_anchor - 1), 128 threads; block y = pair j - 1.
 template <bool FULL>
 __global__ void __launch_bounds__(128) k_par_transport(const __grid_constant__ ParKArgs a) {
   __shared__ float s_zw[kNV];
   __shared__ float s_th[kNB], s_g[kNB], s_own_th[kNB];
   __shared__ int s_own_rel[kNB];
   __shared__ BinInfo s_bins;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tid = threadIdx.x;
   const int tile = blockIdx.x, j = blockIdx.y + 1, tg = a.tile_base + tile;
-  const int t = a.pair_tbeg[j] + (int)blockIdx.z;   // this block's target
-  if (!(a.pair_tbeg[j + 1] > t)) {   // no (further) target: no record
+  if (!(a.pair_tbeg[j + 1] > a.pair_tbeg[j])) {   // no target: no record
     launch_dependents();
     return;
   }
@@ -728,73 +997,139 @@ __global__ void __launch_bounds__(128) k_par_transport(const __grid_constant__ P
       k = (src > 0 ? src : -src) - 1;
       sign = src < 0 ? -1 : 1;
     }
-    float sum = 0.f;
-    if (k >= 0) {
-      // chunk order; twelve loads in flight per round
-      const float* r = a.rec + ((int64_t)tg * a.n_anchor + j) * a.n_chunk * kRec + k;
-      for (int ch0 = 0; ch0 < a.n_chunk; ch0 += 12) {
-        float v[12];
-#pragma unroll
-        for (int u = 0; u < 12; ++u) v[u] = ch0 + u < a.n_chunk ? __ldcg(r + (int64_t)(ch0 + u) * kRec) : 0.f;
-#pragma unroll
-        for (int u = 0; u < 12; ++u) sum += v[u];
-      }
-    }
+    const float sum =
+        k >= 0 ? record_sum(a.rec + ((int64_t)tg * a.n_anchor + j) * a.n_chunk * kRec + k, a.n_chunk) : 0.f;
     s_zw[tid] = sign < 0 ? -sum : sum;
   }
   __syncthreads();
-  if (warp == 0) tile_transport(a, g, s_bins, s_zw, s_th, s_g, s_own_th, s_own_rel, lane);
+  if (tid < 32) tile_transport(a, g, s_bins, s_zw, s_th, s_g, s_own_th, s_own_rel, tid);
   __syncthreads();
-  if (tid < kNB && blockIdx.z == 0) {
+  if (tid < kNB) {
     float* tr = a.trans + ((int64_t)tg * a.n_anchor + j) * 2 * kNB;
     tr[tid] = s_th[tid];
     tr[kNB + tid] = s_g[tid];
   }
-  if (a.img) build_blend_images<FULL>(a, g, s_bins, s_th, s_g, tg, t, t + 1, tid);
-  // the blend is released only now: a tensor-core blend CTA takes a whole SM's shared memory,
-  // and released early it would leave room for too few of this grid's blocks
   launch_dependents();
 }
 
 // ------------------------------------------------------------------ K_blend_tc (bf16)
-// Persistent, one CTA per SM over the (tile, 128-channel chunk) items of one tile kind, 224
-// threads: warp 0 streams the anchors of each item ([8 x 8 tokens][channels] through a
-// 128-byte-swizzled TMA box, the MN-major UMMA operand) through four stages (an item's first
-// anchors load while the previous item's last pairs run); warp 6 streams
-// the blend matrices K_transport wrote, two targets of one pair stacked per group (rows 0-63
-// target 1, 64-127 target 2 of the M = 128 operand), two groups in flight;
-// warp 1 issues one UMMA chain per group (2 pieces x 8 K-steps, M = 128, N = 128) into one of
-// two TMEM buffers; warps 2-5 (one TMEM lane quadrant each: a target slot and 32 output tokens)
-// convert the result to bf16 into a swizzled staging tile that one thread stores with TMA.
-constexpr int kTbNC = 128;                      // channels per item
-constexpr int kTbStages = 4;                    // 225 KB of shared memory in all
-constexpr int kTbPlane = 64 * kTbNC * 2;        // one anchor tile, 16 KB
-constexpr int kTbPiece = 128 * 128 * 2;         // one bf16 piece of a group's [128][128] operand, 32 KB
-constexpr int kTbGroup = 2 * kTbPiece;          // both pieces, 64 KB
-constexpr int kTbOut = 2 * kTbPlane;            // two targets' output tiles, 32 KB
-constexpr int kTbThreads = 224;
-constexpr int kTbSmem = kTbStages * kTbPlane + 2 * kTbGroup + kTbOut + 1024;
+// Persistent, one CTA per SM, 512 threads.  A unit is one (tile, group of up to two targets of a
+// pair) with a range of 128-channel chunks: its blend matrices (two targets stacked into the
+// M = 128 operand, rows 0-63 and 64-127; two bf16 pieces) stay in TMEM while the chunks stream
+// past, [H_t1 ; H_t2] [X_a ; X_b] per chunk (2 pieces x 8 K-steps, N = 128):
+//   warp 0       X_a and X_b of each chunk (TMA, [8 x 8 tokens][channels], the MN-major operand),
+//                four stages of 32 KB
+//   warp 2       the transport of each unit (records -> theta, g), one unit ahead
+//   warps 12..15 the matrices: the convolution kernels h of the unit's targets, a table of their
+//                128 distinct 16-byte rows each, and from it one operand row per thread into TMEM
+//                (two pieces of 64 columns, two units' worth), one unit ahead of the UMMAs
+//   warps 1, 3   UMMA issuers (converged), alternate chunks, A from TMEM, D in one of two 128-column
+//                TMEM buffers
+//   warps 4..11  epilogue: two sets of four warps take alternate chunks; a warp converts 32 output
+//                tokens x 64 channels at a time into one of its two 4 KB staging tiles, which it
+//                stores with TMA by itself (no barrier between warps).
+// Bound by the tensor pipe (1,088 cycles a chunk) and the output stream.  A kernel of its own for
+// the transport, which wrote 32 KB of matrices per (tile, target), and a blend that loaded them
+// for every (tile, chunk) - 64 KB per 32 KB of output through the ~50 bytes per clock that an SM
+// takes from L2, one staging tile for all warps - took 11 and 68 us for the full tiles of the
+// HY-World-shaped call, 9.5 and 19 us beside them for the edge tiles.  With the matrices in shared
+// memory the UMMAs read both operands from there (128 bytes per clock, as much as an SM has).
+constexpr int kTbStages = 4;
+constexpr int kTbPlane = 64 * 128 * 2;          // one anchor tile of a chunk, 16 KB
+constexpr int kTbStage = 2 * kTbPlane;          // X_a and X_b
+constexpr int kTbOut = 32 * 128;                // a warp's 32 tokens x 64 channels
+constexpr int kTbThreads = 512;
+constexpr int kTbMat = 128, kTbD = 256;         // TMEM columns: matrices of unit k at (k & 1) * 128, D buffers at 256
 
-template <bool FULL>
+// The transport of one unit, by one warp.
+struct TransportShared {
+  BinInfo bins;
+  float zw[kNV], own_th[kNB];
+  int own_rel[kNB];
+  unsigned char slot[kNB];
+};
+__device__ void transport_shape(const ParKArgs& a, const TileGeom& g, TransportShared& m, int lane) {
+#pragma unroll 1
+  for (int b = lane; b < kNB; b += 32) {
+    bin_info(a, g, m.bins, b);
+    m.slot[b] = a.bin_slot[tile_shape(a, g)][b];
+  }
+  __syncwarp();
+}
+__device__ void unit_transport(const ParKArgs& a, const TileGeom& g, int tile, int j, TransportShared& m, float* th,
+                               float* gate, int lane) {
+  const float* rec = a.rec + ((int64_t)tile * a.n_anchor + j) * a.n_chunk * kRec;
+  // four entries per lane, summed over the parts in order, sixteen loads in flight
+  constexpr int kPer = (kNV + 31) / 32;
+  int at[kPer];
+  float sum[kPer];
+#pragma unroll
+  for (int i = 0; i < kPer; ++i) {
+    const int e = lane + 32 * i, b = min(e / 3, kNB - 1), comp = e - 3 * (e / 3), code = m.slot[b], slot = code & 63;
+    // Re Z, Im Z, W of complex slot s stand at s, 30 + s, 60 + s, Z and W of real slot s at 90 + s, 94 + s
+    at[i] = comp * kNCpx + slot;
+    if (code & kSlotReal) at[i] = comp == 1 ? -1 : 3 * kNCpx + (comp == 2 ? kNReal : 0) + slot;
+    if (code == 255 || e >= kNV) at[i] = -1;
+    sum[i] = 0.f;
+  }
+  for (int q0 = 0; q0 < a.st_parts; q0 += 4) {
+    float v[kPer][4];
+#pragma unroll
+    for (int i = 0; i < kPer; ++i)
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        v[i][q] = at[i] >= 0 && q0 + q < a.st_parts ? __ldcg(rec + (int64_t)(q0 + q) * kRec + at[i]) : 0.f;
+#pragma unroll
+    for (int i = 0; i < kPer; ++i)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) sum[i] += v[i][q];
+  }
+#pragma unroll
+  for (int i = 0; i < kPer; ++i) {
+    const int e = lane + 32 * i;
+    if (e < kNV) m.zw[e] = (e % 3) == 1 && (m.slot[e / 3] & kSlotMirror) && at[i] >= 0 ? -sum[i] : sum[i];
+  }
+  __syncwarp();
+  tile_transport(a, g, m.bins, m.zw, th, gate, m.own_th, m.own_rel, lane);
+  __syncwarp();
+}
+
+// The matrices of one unit, by 128 threads (barrier 3): thread = (side, dy, xo).
+// Row m = output token 8 yo + xo, column 64 side + 8 yi + xi = input token of anchor a (side 0)
+// or b (side 1); entry h_side((yo - yi) mod h, (xo - xi) mod w) with
+// h_side(d) = (1 / (h w)) sum over stored bins of kappa' Re(phi_side e^{2 pi i (ky dy / h + kx dx / w)}),
+// kappa' = 1 on the kx = 0 and Nyquist columns (every ky stored), 2 elsewhere;
+// phi_a = (1 - alpha) e^{i g alpha theta}, phi_b = alpha e^{-i g (1 - alpha) theta}.  The sum runs
+// over kx first (one complex value per (ky, dx)), then over ky.
+struct MatrixShared {
+  uint4 row[2][2][2][64];   // [target][piece][side][8 dy + xo]: entries (xo - xi) mod w, xi = 0..7, of row dy
+  float4 phi[2][kNB];
+  float2 col[2][2][64];     // [target][side][8 ky + dx]
+  float h[2][2][64];        // [target][side][8 dy + dx]
+};
+constexpr int kTbSmem = kTbStages * kTbStage + 16 * kTbOut + (int)sizeof(MatrixShared) + 1024;
+
+__device__ __forceinline__ void matrix_sync() { asm volatile("bar.sync 3, 128;" ::: "memory"); }
+
 __global__ void __launch_bounds__(kTbThreads, 1)
     k_par_blend_tc(const __grid_constant__ CUtensorMap tm, const __grid_constant__ CUtensorMap tm_out,
-                   const __grid_constant__ ParKArgs a, int n_tiles) {
+                   const __grid_constant__ ParKArgs a) {
   extern __shared__ uint8_t dsm_raw[];
   const uint32_t raw_addr = smem_u32(dsm_raw);
   uint8_t* dsm = dsm_raw + (((raw_addr + 1023u) & ~1023u) - raw_addr);   // 128-byte swizzle atoms
-  uint8_t* s_stage = dsm;
-  uint8_t* s_img = dsm + kTbStages * kTbPlane;
-  uint8_t* s_out = s_img + 2 * kTbGroup;
-  __shared__ __align__(8) uint64_t b_full[kTbStages], b_empty[kTbStages], b_ifull[2], b_iempty[2],
-      b_tfull[2], b_tempty[2];
+  uint8_t* s_x = dsm;
+  uint8_t* s_out = dsm + kTbStages * kTbStage;
+  MatrixShared& m = *reinterpret_cast<MatrixShared*>(s_out + 16 * kTbOut);
+  __shared__ __align__(8) uint64_t b_xfull[kTbStages], b_xempty[kTbStages], b_mfull[2], b_mempty[2], b_dfull[2],
+      b_dempty[2], b_tready, b_tfree;
+  __shared__ float s_th[kNB], s_gate[kNB];   // of the unit whose matrices are next
   __shared__ uint32_t s_tmem;
   __shared__ volatile int s_abort;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int n_anc = a.n_anchor;
-  const int nck = (a.C + kTbNC - 1) / kTbNC;   // 128-channel chunks per tile
-  const int n_items = nck * n_tiles;           // item = tile * nck + chunk, CTAs stride the items
+  const int n_units = a.n_tile * a.n_grp * a.bl_parts;
   const uint64_t lim = a.wait_ns;
   auto wait = [&](uint64_t* bar, uint32_t parity) -> bool {
+    if (mbar_try_wait(bar, parity)) return true;
     if (s_abort) return false;
     if (mbar_wait(bar, parity, lim)) return true;
     s_abort = 1;
@@ -803,186 +1138,307 @@ __global__ void __launch_bounds__(kTbThreads, 1)
   };
   if (tid == 0) {
     for (int s = 0; s < kTbStages; ++s) {
-      mbar_init(&b_full[s], 1);
-      mbar_init(&b_empty[s], 1);
+      mbar_init(&b_xfull[s], 1);
+      mbar_init(&b_xempty[s], 1);
     }
     for (int b = 0; b < 2; ++b) {
-      mbar_init(&b_ifull[b], 1);
-      mbar_init(&b_iempty[b], 1);
-      mbar_init(&b_tfull[b], 1);
-      mbar_init(&b_tempty[b], 4);
+      mbar_init(&b_mfull[b], 128);
+      mbar_init(&b_mempty[b], 2);   // both issuers
+      mbar_init(&b_dfull[b], 1);
+      mbar_init(&b_dempty[b], 4);
     }
+    mbar_init(&b_tready, 1);
+    mbar_init(&b_tfree, 1);
     fence_barrier_init();
     s_abort = 0;
   }
   if (warp == 1) {
-    tmem_alloc(&s_tmem, 2 * kTbNC);
+    tmem_alloc(&s_tmem, 512);
     tmem_relinquish();
+    tc_fence_before();
   }
-  launch_dependents();
-  // the blend images come from the preceding K_transport (and the anchors from kernels before)
-  grid_dependency_wait();
-  tc_fence_before();
+  zero_stages(a, s_x, kTbStages * kTbStage);
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = s_tmem;
-  constexpr uint32_t kAnchorBytes = (uint32_t)kTbPlane;
+  // (only the transport reads what K_stats_tc wrote: its warp waits for that grid)
+  // unit u -> (tile, target group, chunk range): groups innermost, so that a tile's anchors are
+  // read from L2 by the CTAs of neighbouring units
+  struct Unit {
+    int tile, grp, c0, c1;
+  };
+  auto unit_of = [&](int u) {
+    Unit x;
+    const int per = a.n_grp * a.bl_parts;
+    x.tile = u / per;
+    const int r = u - x.tile * per, part = r / a.n_grp;
+    x.grp = r - part * a.n_grp;
+    x.c0 = part * a.bl_cpp;
+    x.c1 = min(a.n_chunk, x.c0 + a.bl_cpp);
+    return x;
+  };
 
   if (warp == 0) {
-    // ---------------------------------------------------------------- anchor producer
-    // anchor load L (counted over the CTA's items) goes into stage L % kTbStages once anchor
-    // L - kTbStages has been released by the UMMA issuer
     if (lane == 0) {
+      // -------------------------------------------------------------- anchor producer
       tma_prefetch_desc(&tm);
-      int L = 0;
-      for (int item = blockIdx.x; item < n_items && !s_abort; item += gridDim.x) {
-        const int tile = item / nck, c0 = (item - tile * nck) * kTbNC;
-        const TileGeom g = tile_geom(a, tile, FULL);
-        for (int i = 0; i < n_anc; ++i, ++L) {
-          const int s = L % kTbStages;
-          if (L >= kTbStages && !wait(&b_empty[s], (uint32_t)((L / kTbStages) - 1) & 1u)) break;
-          mbar_arrive_expect_tx(&b_full[s], kAnchorBytes);
-          tma_load_4d(s_stage + s * kTbPlane, &tm, &b_full[s], c0, g.x0, g.y0, a.anchor_frame[i]);
-          tma_load_4d(s_stage + s * kTbPlane + 8192, &tm, &b_full[s], c0 + 64, g.x0, g.y0, a.anchor_frame[i]);
-        }
-      }
-      if (s_abort)   // the copies still in flight land before the shared memory is released
-        for (int l = L > kTbStages ? L - kTbStages : 0; l < L; ++l)
-          mbar_wait(&b_full[l % kTbStages], (uint32_t)(l / kTbStages) & 1u, lim);
-    }
-  } else if (warp == 6) {
-    // ---------------------------------------------------------------- image producer
-    if (lane == 0) {
       int n = 0;
-      for (int item = blockIdx.x; item < n_items && !s_abort; item += gridDim.x) {
-        const int tg = a.tile_base + item / nck;
-        for (int j = 1; j < n_anc && !s_abort; ++j)
-          for (int t0 = a.pair_tbeg[j]; t0 < a.pair_tbeg[j + 1]; t0 += 2, ++n) {
-            const int ib = n & 1, nt = min(2, a.pair_tbeg[j + 1] - t0);
-            if (n >= 2 && !wait(&b_iempty[ib], (uint32_t)((n >> 1) - 1) & 1u)) break;
-            mbar_arrive_expect_tx(&b_ifull[ib], (uint32_t)(nt * kImgBytes));
-            uint8_t* dst = s_img + ib * kTbGroup;
-            for (int ts = 0; ts < nt; ++ts) {
-              const char* src = a.img + ((int64_t)tg * a.n_target + t0 + ts) * kImgBytes;
-              // piece p, K-block kb of the target -> rows 64 ts .. 64 ts + 63 of the stacked operand
-              for (int p = 0; p < 2; ++p)
-                for (int kb = 0; kb < 2; ++kb)
-                  bulk_load(dst + p * kTbPiece + kb * 16384 + ts * 8192, src + p * kImgTerm + kb * 8192, 8192u,
-                            &b_ifull[ib]);
-            }
-          }
-      }
-      if (s_abort)   // let the images in flight land (at most the last two groups)
-        for (int l = n > 2 ? n - 2 : 0; l < n; ++l) mbar_wait(&b_ifull[l & 1], (uint32_t)(l >> 1) & 1u, lim);
-    }
-  } else if (warp == 1) {
-    // ---------------------------------------------------------------- UMMA issuer
-    if (lane == 0) {
-      const uint32_t idesc = idesc_bf16_f32(128, kTbNC, false, true);
-      int n = 0, L = 0;
       bool ok = true;
-      for (int item = blockIdx.x; ok && item < n_items; item += gridDim.x, L += n_anc) {
-        if (!wait(&b_full[L % kTbStages], (uint32_t)(L / kTbStages) & 1u)) break;
-        for (int j = 1; ok && j < n_anc; ++j) {
-          const int La = L + j - 1, Lb = L + j;
-          if (!wait(&b_full[Lb % kTbStages], (uint32_t)(Lb / kTbStages) & 1u)) { ok = false; break; }
-          const uint32_t xa = smem_u32(s_stage + (La % kTbStages) * kTbPlane);
-          const uint32_t xb = smem_u32(s_stage + (Lb % kTbStages) * kTbPlane);
-          for (int t0 = a.pair_tbeg[j]; t0 < a.pair_tbeg[j + 1]; t0 += 2, ++n) {
-            const int ib = n & 1;
-            if (!wait(&b_ifull[ib], (uint32_t)(n >> 1) & 1u) ||
-                (n >= 2 && !wait(&b_tempty[ib], (uint32_t)((n >> 1) - 1) & 1u))) { ok = false; break; }
-            tc_fence_after();
-            const uint32_t im = smem_u32(s_img + ib * kTbGroup), d = tmem + (uint32_t)(ib * kTbNC);
-#pragma unroll
-            for (int p = 0; p < 2; ++p)
-#pragma unroll
-              for (int kk = 0; kk < 8; ++kk)
-                umma_bf16_ss(d, sdesc_sw128(im + p * kTbPiece + (kk >> 2) * 16384 + (kk & 3) * 32, 16, 1024),
-                             sdesc_sw128((kk < 4 ? xa : xb) + (kk & 3) * 2048, 8192, 1024), idesc,
-                             (p | kk) ? 1u : 0u);
-            umma_commit(&b_iempty[ib]);
-            umma_commit(&b_tfull[ib]);
-          }
-          if (ok) umma_commit(&b_empty[La % kTbStages]);   // the pair's UMMAs were anchor La's last readers
+      for (int u = blockIdx.x; ok && u < n_units; u += gridDim.x) {
+        const Unit x = unit_of(u);
+        const TileGeom g = any_tile(a, x.tile);
+        const int j = a.grp_pair[x.grp];
+        for (int c = x.c0; c < x.c1; ++c, ++n) {
+          const int s = n % kTbStages;
+          if (n >= kTbStages && !wait(&b_xempty[s], (uint32_t)((n / kTbStages) - 1) & 1u)) { ok = false; break; }
+          mbar_arrive_expect_tx(&b_xfull[s], 2 * anchor_tile_bytes(a));
+          for (int q = 0; q < 2; ++q)
+            load_anchor_tile(a, &tm, s_x + s * kTbStage + q * kTbPlane, &b_xfull[s], c * 128, g, a.anchor_frame[j - 1 + q]);
         }
-        if (ok) umma_commit(&b_empty[(L + n_anc - 1) % kTbStages]);   // the item's last anchor
       }
-      if (s_abort && n > 0) mbar_wait(&b_tfull[(n - 1) & 1], (uint32_t)((n - 1) >> 1) & 1u, lim);
+      if (!ok)   // the copies still in flight land before the shared memory is released
+        for (int l = n > kTbStages ? n - kTbStages : 0; l < n; ++l)
+          mbar_wait(&b_xfull[l % kTbStages], (uint32_t)(l / kTbStages) & 1u, lim);
     }
-  } else if (warp >= 2 && warp <= 5) {
-    // ---------------------------------------------------------------- epilogue warps 2-5
-    // (warp 6 has no role: it goes straight to the final barrier)
-    const int ctid = tid - 64;                 // 0..127
-    const int q = warp & 3;                    // TMEM lanes 32 q .. 32 q + 31
-    const int ts = q >> 1;                     // target slot of this warp
-    const int o = 32 * (q & 1) + lane;         // output token 8 y + x
-    const int yo = o >> 3, xo = o & 7;
-    const bool valid = yo < a.th && xo < a.tw;
-    const int sr = yo * a.tw + xo;             // row inside the store box
-    uint8_t* out = s_out + ts * kTbPlane;
-    bool fail = false;
+  } else if (warp >= 12) {
+    // ---------------------------------------------------------------- matrices
+    const int mt = tid - 384, side = mt >> 6, dy = (mt >> 3) & 7, dx = mt & 7;   // dy also ky, dx also xo
+    // this thread's operand row (TMEM lane): target slot and output token
+    const int rts = mt >> 6, ryo = (mt >> 3) & 7, rxo = mt & 7;
+    const uint32_t tm = tmem + ((uint32_t)((warp & 3) * 32) << 16);
+    int k = 0, shape = -1;
+    float2 twx[5], twy[8];   // e^{2 pi i kx dx / w}, e^{2 pi i ky dy / h}; 0 past the stored bins
+    for (int u = blockIdx.x; u < n_units; u += gridDim.x, ++k) {
+      const Unit x = unit_of(u);
+      const TileGeom g = any_tile(a, x.tile);
+      const int h = g.h, w = g.w, t0 = a.grp_t0[x.grp], nt = a.grp_nt[x.grp];
+      if (h * 16 + w != shape) {
+        shape = h * 16 + w;
+#pragma unroll
+        for (int q = 0; q < 5; ++q) {
+          float sv, cv;
+          sincospif(2.f * (float)(q * dx % w) / (float)w, &sv, &cv);
+          twx[q] = q <= w / 2 ? make_float2(cv, sv) : make_float2(0.f, 0.f);
+        }
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+          float sv, cv;
+          sincospif(2.f * (float)(q * dy % h) / (float)h, &sv, &cv);
+          twy[q] = q < h ? make_float2(cv, sv) : make_float2(0.f, 0.f);
+        }
+      }
+      // (the four warps leave together)
+      if (bar_sync_or(3, 128, !wait(&b_tready, (uint32_t)k & 1u))) break;
+      if (mt < 2 * kNB) {
+        const int ts = mt / kNB, b = mt - ts * kNB, ky = b / 5, kx = b % 5;
+        float4 ph = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (ts < nt && ky < h && kx <= w / 2) {
+          const float al = a.target_alpha[t0 + ts];
+          const bool edge = kx == 0 || ((w % 2 == 0) && kx == w / 2);
+          const float kap = (edge ? 1.f : 2.f) / (float)(h * w);
+          float sa, ca, sb, cb;
+          const float gt = s_gate[b] * s_th[b];
+          sincosf(gt * al, &sa, &ca);
+          sincosf(-gt * (1.f - al), &sb, &cb);
+          ph = make_float4(kap * (1.f - al) * ca, kap * (1.f - al) * sa, kap * al * cb, kap * al * sb);
+        }
+        m.phi[ts][b] = ph;
+      }
+      matrix_sync();
+      if (mt == 0) mbar_arrive(&b_tfree);   // theta and g have been read
+#pragma unroll
+      for (int ts = 0; ts < 2; ++ts) {
+        float cr = 0.f, ci = 0.f;
+#pragma unroll
+        for (int kx = 0; kx < 5; ++kx) {
+          const float4 ph = m.phi[ts][dy * 5 + kx];
+          const float pr = side ? ph.z : ph.x, pi = side ? ph.w : ph.y;
+          cr = fmaf(pr, twx[kx].x, fmaf(-pi, twx[kx].y, cr));
+          ci = fmaf(pr, twx[kx].y, fmaf(pi, twx[kx].x, ci));
+        }
+        m.col[ts][side][dy * 8 + dx] = make_float2(cr, ci);
+      }
+      matrix_sync();
+#pragma unroll
+      for (int ts = 0; ts < 2; ++ts) {
+        float acc = 0.f;
+#pragma unroll
+        for (int ky = 0; ky < 8; ++ky) {
+          const float2 c = m.col[ts][side][ky * 8 + dx];
+          acc = fmaf(c.x, twy[ky].x, fmaf(-c.y, twy[ky].y, acc));
+        }
+        m.h[ts][side][dy * 8 + dx] = acc;
+      }
+      matrix_sync();
+      // the distinct rows of 8 input columns in two bf16 pieces
+#pragma unroll
+      for (int ts = 0; ts < 2; ++ts) {
+        uint32_t hi[4], lo[4];
+#pragma unroll
+        for (int xi = 0; xi < 8; xi += 2) {
+          float v[2];
+#pragma unroll
+          for (int q = 0; q < 2; ++q) {
+            const int d = dx - xi - q + (dx < xi + q ? w : 0);
+            v[q] = dy < h && dx < w && xi + q < w ? m.h[ts][side][dy * 8 + d] : 0.f;
+          }
+          const __nv_bfloat162 b1 = __floats2bfloat162_rn(v[0], v[1]);
+          const __nv_bfloat162 b2 = __floats2bfloat162_rn(v[0] - __low2float(b1), v[1] - __high2float(b1));
+          hi[xi / 2] = *reinterpret_cast<const uint32_t*>(&b1);
+          lo[xi / 2] = *reinterpret_cast<const uint32_t*>(&b2);
+        }
+        m.row[ts][0][side][dy * 8 + dx] = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+        m.row[ts][1][side][dy * 8 + dx] = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+      }
+      // the UMMAs of the unit before the last have read their matrices
+      const int mb = k & 1;
+      if (bar_sync_or(3, 128, k >= 2 && !wait(&b_mempty[mb], (uint32_t)((k >> 1) - 1) & 1u))) break;
+      tc_fence_after();
+#pragma unroll
+      for (int p = 0; p < 2; ++p)
+#pragma unroll
+        for (int sd = 0; sd < 2; ++sd) {
+          uint32_t v[32];
+#pragma unroll
+          for (int yi = 0; yi < 8; ++yi) {
+            const int d = ryo - yi + (ryo < yi ? h : 0);
+            uint4 q = make_uint4(0u, 0u, 0u, 0u);
+            if (yi < h && ryo < h) q = m.row[rts][p][sd][d * 8 + rxo];
+            v[4 * yi] = q.x;
+            v[4 * yi + 1] = q.y;
+            v[4 * yi + 2] = q.z;
+            v[4 * yi + 3] = q.w;
+          }
+          tmem_st_x32_async(tm + (uint32_t)(mb * kTbMat + p * 64 + sd * 32), v);
+        }
+      tmem_wait_st();
+      tc_fence_before();
+      mbar_arrive(&b_mfull[mb]);
+    }
+  } else if (warp == 2) {
+    // ---------------------------------------------------------------- transport
+    __shared__ TransportShared ms;
+    int k = 0, shape = -1;
+    for (int u = blockIdx.x; u < n_units; u += gridDim.x, ++k) {
+      const Unit x = unit_of(u);
+      const TileGeom g = any_tile(a, x.tile);
+      const bool fresh = g.h * 16 + g.w != shape;
+      shape = g.h * 16 + g.w;
+      if (fresh) transport_shape(a, g, ms, lane);
+      if (k == 0) grid_dependency_wait();   // the records of K_stats_tc
+      if (!__all_sync(0xffffffffu, k == 0 || wait(&b_tfree, (uint32_t)(k - 1) & 1u))) break;
+      unit_transport(a, g, x.tile, a.grp_pair[x.grp], ms, s_th, s_gate, lane);
+      if (lane == 0) mbar_arrive(&b_tready);
+    }
+  } else if (warp < 4) {
+    // ---------------------------------------------------------------- UMMA issuers (converged)
+    // warps 1 and 3 take alternate chunks and accumulators (see K_stats_tc)
+    constexpr uint32_t idesc = idesc_bf16_f32(128, 128, false, true);
+    const int buf = warp >> 1;
+    const uint32_t tmu = __shfl_sync(0xffffffffu, tmem, 0);
+    const uint32_t xb = __shfl_sync(0xffffffffu, smem_u32(s_x), 0);
+    const uint64_t dx = sdesc_sw128(xb, 8192, 1024);
+    const bool lead = elect_one();
+    int n = 0, k = 0, last = -1;
+    bool ok = true;
+    for (int u = blockIdx.x; ok && u < n_units; u += gridDim.x, ++k) {
+      const Unit x = unit_of(u);
+      const int mb = k & 1;
+      if (!(ok = __all_sync(0xffffffffu, wait(&b_mfull[mb], (uint32_t)(k >> 1) & 1u)))) break;
+      tc_fence_after();
+      for (int c = x.c0; c < x.c1; ++c, ++n) {
+        if ((n & 1) != buf) continue;
+        const int s = n % kTbStages;
+        // half of the warp waits for the anchors, half for the accumulator
+        const bool w = lane < 16 ? wait(&b_xfull[s], (uint32_t)(n / kTbStages) & 1u)
+                                 : n < 2 || wait(&b_dempty[buf], (uint32_t)((n >> 1) - 1) & 1u);
+        if (!(ok = __all_sync(0xffffffffu, w))) break;
+        tc_fence_after();
+        if (lead) {
+          const uint64_t db = dx + (uint64_t)(s * (kTbStage >> 4));
+#pragma unroll
+          for (int p = 0; p < 2; ++p)
+#pragma unroll
+            for (int kk = 0; kk < 8; ++kk)
+              umma_bf16_ts(tmu + (uint32_t)(kTbD + buf * 128), tmu + (uint32_t)(mb * kTbMat + p * 64 + kk * 8),
+                           db + (uint64_t)(((kk >> 2) * kTbPlane + (kk & 3) * 2048) >> 4), idesc, (p | kk) ? 1u : 0u);
+          umma_commit(&b_xempty[s]);
+          umma_commit(&b_dfull[buf]);
+        }
+        __syncwarp();
+        last = n;
+      }
+      // this issuer's last reads of the unit's matrices
+      if (ok && lead) umma_commit(&b_mempty[mb]);
+      __syncwarp();
+    }
+    // the UMMAs issued so far have completed before shared memory and TMEM are released
+    if (last >= 0) mbar_wait(&b_dfull[buf], (uint32_t)(last >> 1) & 1u, lim);
+    __syncwarp();
+  } else if (warp >= 4) {   // 4..11
+    // ---------------------------------------------------------------- epilogue
+    const int set = (warp - 4) >> 2, q = warp & 3;   // TMEM lanes 32 q .. 32 q + 31
+    const int ts = q >> 1;                           // target slot of this warp
+    const int o = 32 * (q & 1) + lane, yo = o >> 3, xo = o & 7;   // output token 8 y + x
+    const bool valid = yo < a.th && xo < a.tw, whole = a.th == 8 && a.tw == 8;
+    uint8_t* out0 = s_out + (warp - 4) * 2 * kTbOut;   // two tiles, row yo & 3 at 1 KB each
+    const int doff = (yo & 3) * 1024 + xo * 128;
     int n = 0;
-    for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
-      const int tile = item / nck, c0 = (item - tile * nck) * kTbNC;
-      const TileGeom g = tile_geom(a, tile, FULL);
-      for (int j = 1; j < n_anc; ++j)
-        for (int t0 = a.pair_tbeg[j]; t0 < a.pair_tbeg[j + 1]; t0 += 2, ++n) {
-          const int ib = n & 1, nt = min(2, a.pair_tbeg[j + 1] - t0);
-          if (!fail && !wait(&b_tfull[ib], (uint32_t)(n >> 1) & 1u)) fail = true;
-          // the previous group's TMA stores have read the staging tiles
-          if (ctid == 0) bulk_wait_read_all();
-          if (bar_sync_or(1, 128, fail)) {
-            fail = true;
+    bool ok = true;
+    for (int u = blockIdx.x; ok && u < n_units; u += gridDim.x) {
+      const Unit x = unit_of(u);
+      const TileGeom g = any_tile(a, x.tile);
+      const bool mine = ts < a.grp_nt[x.grp];
+      const int frame = mine ? a.target_frame[a.grp_t0[x.grp] + ts] : 0, y0 = g.y0 + 4 * (q & 1);
+      for (int c = x.c0; c < x.c1; ++c, ++n) {
+        if ((n & 1) != set) continue;
+        if (!__all_sync(0xffffffffu, wait(&b_dfull[set], (uint32_t)(n >> 1) & 1u))) { ok = false; break; }
+        tc_fence_after();
+        const uint32_t ta = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(kTbD + set * 128);
+#pragma unroll
+        for (int half = 0; half < 2; ++half) {
+          // 64 channels (one 128-byte box) at a time
+          uint32_t r[64];
+          tmem_ld_x64(ta + 64 * half, r);
+          if (half == 1) {   // the whole buffer is in registers: it goes back to the issuer
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive(&b_tempty[ib]);
-            continue;
+            if (lane == 0) mbar_arrive(&b_dempty[set]);
           }
-          tc_fence_after();
-          const uint32_t ta = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(ib * kTbNC);
+          uint32_t pk[32];
 #pragma unroll
-          for (int half = 0; half < 2; ++half) {
-            // 64 channels (one 128-byte box) at a time
-            uint32_t r[64];
-            tmem_ld_x64(ta + 64 * half, r);
-            if (half == 1) {   // the whole buffer is in registers: it goes back to the issuer
-              tc_fence_before();
-              __syncwarp();
-              if (lane == 0) mbar_arrive(&b_tempty[ib]);
-            }
-            if (ts < nt && valid) {
-#pragma unroll
-              for (int c8 = 0; c8 < 8; ++c8) {
-                uint32_t pk[4];
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                  const __nv_bfloat162 b2 = __floats2bfloat162_rn(__uint_as_float(r[8 * c8 + 2 * u]),
-                                                                  __uint_as_float(r[8 * c8 + 2 * u + 1]));
-                  pk[u] = *reinterpret_cast<const uint32_t*>(&b2);
-                }
-                *reinterpret_cast<uint4*>(out + half * 8192 + sr * 128 + ((c8 ^ (sr & 7)) << 4)) =
-                    make_uint4(pk[0], pk[1], pk[2], pk[3]);
-              }
-            }
+          for (int e = 0; e < 32; ++e) {
+            const __nv_bfloat162 b2 = __floats2bfloat162_rn(__uint_as_float(r[2 * e]), __uint_as_float(r[2 * e + 1]));
+            pk[e] = *reinterpret_cast<const uint32_t*>(&b2);
           }
+          uint8_t* out = out0 + half * kTbOut;
+          if (lane == 0) bulk_wait_read_1();   // the store before the last has read this tile
+          __syncwarp();
+          if (mine && valid)
+#pragma unroll
+            for (int c8 = 0; c8 < 8; ++c8)
+              *reinterpret_cast<uint4*>(out + doff + ((c8 ^ xo) << 4)) =
+                  make_uint4(pk[4 * c8], pk[4 * c8 + 1], pk[4 * c8 + 2], pk[4 * c8 + 3]);
           fence_proxy_async_smem();
-          bar_sync_or(1, 128, false);
-          if (ctid == 0) {
-            for (int u = 0; u < nt; ++u)
-              for (int b = 0; b < 2; ++b)
-                if (c0 + 64 * b < a.C)
-                  tma_store_4d(&tm_out, s_out + u * kTbPlane + b * 8192, c0 + 64 * b, g.x0, g.y0,
-                               a.target_frame[t0 + u]);
-            bulk_commit();
+          __syncwarp();
+          const int ch = c * 128 + 64 * half;
+          if (lane == 0) {
+            if (mine && ch < a.C && whole) {   // four rows of eight tokens
+              if (y0 < a.Hg) tma_store_4d(&tm_out, out, ch, g.x0, y0, frame);
+            } else if (mine && ch < a.C) {     // smaller tiles: one row at a time
+              for (int yy = 4 * (q & 1); yy < min(a.th, 4 * (q & 1) + 4) && g.y0 + yy < a.Hg; ++yy)
+                tma_store_4d(&tm_out, out + (yy & 3) * 1024, ch, g.x0, g.y0 + yy, frame);
+            }
+            bulk_commit();   // one group per half, also where nothing is stored
           }
         }
+      }
     }
-    if (ctid == 0) bulk_wait_all();
+    if (lane == 0) bulk_wait_all();
   }
   tc_fence_before();
   __syncthreads();
-  if (warp == 1) tmem_dealloc(tmem, 2 * kTbNC);
+  if (warp == 1) tmem_dealloc(tmem, 512);
 }
 
 // 4-D map [F][Hg][Wg][C] with a 128-byte-swizzled box (64 bf16 channels, bw, bh, 1)
@@ -1012,19 +1468,50 @@ bool make_r_map(CUtensorMap* m, const cast_par_args& a, int cc) {
             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// One tile kind on one stream: K_stats, then K_transport and K_blend as programmatic dependents.
-template <typename T, bool FULL>
-cast_status launch_kind(const CUtensorMap& tm, const CUtensorMap* tm_sw, const CUtensorMap* tm_out,
-                        const ParKArgs& k, int n_tiles, cudaStream_t st) {
-  const size_t smem = par_dyn_smem<T>(kCC);
+// bf16: two launches over every tile, the second a programmatic dependent of the first.
+cast_status launch_tc(const CUtensorMap& tm_sw, const CUtensorMap& tm_out, const ParKArgs& k, cudaStream_t st) {
+  static std::atomic<uint64_t> attr_done{0};
+  if (!once_per_device(attr_done, [] {
+        return cudaFuncSetAttribute(k_par_stats_tc<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kStSmem) ==
+                   cudaSuccess &&
+               cudaFuncSetAttribute(k_par_stats_tc<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kStSmem) ==
+                   cudaSuccess &&
+               cudaFuncSetAttribute(k_par_blend_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, kTbSmem) ==
+                   cudaSuccess;
+      }))
+    return check_launch("PAR kernel attributes");
+  const int nsm = sm_count();
+  cudaLaunchAttribute pdl[1];
+  pdl[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  pdl[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(std::min(k.n_tile * k.n_act * k.st_parts, nsm), 1, 1);
+  cfg.blockDim = dim3(kStThreads, 1, 1);
+  cfg.dynamicSmemBytes = kStSmem;
+  cfg.stream = st;
+  if (cudaLaunchKernelEx(&cfg, k.wch ? k_par_stats_tc<true> : k_par_stats_tc<false>, tm_sw, k) != cudaSuccess) return check_launch("PAR statistics kernel");
+  cudaLaunchConfig_t bc{};
+  bc.gridDim = dim3(std::min(k.n_tile * k.n_grp * k.bl_parts, nsm), 1, 1);
+  bc.blockDim = dim3(kTbThreads, 1, 1);
+  bc.dynamicSmemBytes = kTbSmem;
+  bc.stream = st;
+  bc.attrs = pdl;
+  bc.numAttrs = 1;
+  if (cudaLaunchKernelEx(&bc, k_par_blend_tc, tm_sw, tm_out, k) != cudaSuccess)
+    return check_launch("PAR tensor-core blend kernel");
+  return check_launch("PAR kernels");
+}
+
+// f32, one tile kind on one stream: K_stats, then K_transport and K_blend as programmatic dependents.
+template <bool FULL>
+cast_status launch_kind(const CUtensorMap& tm, const ParKArgs& k, int n_tiles, cudaStream_t st) {
+  const size_t smem = par_dyn_smem(kCC);
   static std::atomic<uint64_t> attr_done{0};
   if (!once_per_device(attr_done, [smem] {
-        return cudaFuncSetAttribute(k_par<T, kCC, FULL, true>,
-                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess &&
-               cudaFuncSetAttribute(k_par<T, kCC, FULL, false>,
-                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess &&
-               cudaFuncSetAttribute(k_par_blend_tc<FULL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    kTbSmem) == cudaSuccess;
+        return cudaFuncSetAttribute(k_par<kCC, FULL, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)smem) == cudaSuccess &&
+               cudaFuncSetAttribute(k_par<kCC, FULL, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)smem) == cudaSuccess;
       }))
     return check_launch("PAR kernel attributes");
   cudaLaunchAttribute pdl[1];
@@ -1035,13 +1522,10 @@ cast_status launch_kind(const CUtensorMap& tm, const CUtensorMap* tm_sw, const C
   cfg.blockDim = dim3(kCC, 1, 1);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
-  if (cudaLaunchKernelEx(&cfg, k_par<T, kCC, FULL, true>, tm, k) != cudaSuccess)
+  if (cudaLaunchKernelEx(&cfg, k_par<kCC, FULL, true>, tm, k) != cudaSuccess)
     return check_launch("PAR statistics kernel");
-  int zmax = 1;   // one transport block per (tile, pair, target) when it writes blend matrices
-  if (k.img)
-    for (int j = 1; j < k.n_anchor; ++j) zmax = std::max(zmax, k.pair_tbeg[j + 1] - k.pair_tbeg[j]);
   cudaLaunchConfig_t tc{};
-  tc.gridDim = dim3(n_tiles, k.n_anchor - 1, zmax);
+  tc.gridDim = dim3(n_tiles, k.n_anchor - 1, 1);
   tc.blockDim = dim3(128, 1, 1);
   tc.stream = st;
   tc.attrs = pdl;
@@ -1050,23 +1534,8 @@ cast_status launch_kind(const CUtensorMap& tm, const CUtensorMap* tm_sw, const C
     return check_launch("PAR transport kernel");
   cfg.attrs = pdl;
   cfg.numAttrs = 1;
-  if (k.img) {
-    // bf16: the blend as tensor-core GEMMs over the matrices K_transport wrote
-    // persistent: one CTA per SM over the (tile, 128-channel chunk) items of this kind
-    const int nsm = sm_count();
-    const int items = ((k.C + kTbNC - 1) / kTbNC) * n_tiles;
-    cudaLaunchConfig_t bc{};
-    bc.gridDim = dim3(items < nsm ? items : nsm, 1, 1);
-    bc.blockDim = dim3(kTbThreads, 1, 1);
-    bc.dynamicSmemBytes = kTbSmem;
-    bc.stream = st;
-    bc.attrs = pdl;
-    bc.numAttrs = 1;
-    if (cudaLaunchKernelEx(&bc, k_par_blend_tc<FULL>, *tm_sw, *tm_out, k, n_tiles) != cudaSuccess)
-      return check_launch("PAR tensor-core blend kernel");
-  } else if (cudaLaunchKernelEx(&cfg, k_par<T, kCC, FULL, false>, tm, k) != cudaSuccess) {
+  if (cudaLaunchKernelEx(&cfg, k_par<kCC, FULL, false>, tm, k) != cudaSuccess)
     return check_launch("PAR blend kernel");
-  }
   return check_launch("PAR kernels");
 }
 
@@ -1109,23 +1578,21 @@ ParKArgs with_segments(const ParKArgs& k0, int nseg) {
   return k;
 }
 
-template <typename T>
-cast_status launch_typed(const CUtensorMap& tm, const CUtensorMap* tm_sw, const CUtensorMap* tm_out,
-                         const ParKArgs& k0, const ParPlan& p, cudaStream_t st) {
+cast_status launch_f32(const CUtensorMap& tm, const ParKArgs& k0, const ParPlan& p, cudaStream_t st) {
   ParKArgs kf = with_segments(k0, p.n_tseg_full), ke = with_segments(k0, p.n_tseg_edge);
   kf.tile_base = 0;
   ke.tile_base = p.n_full;
-  if (p.n_edge == 0) return launch_kind<T, true>(tm, tm_sw, tm_out, kf, p.n_full, st);
-  if (p.n_full == 0) return launch_kind<T, false>(tm, tm_sw, tm_out, ke, p.n_edge, st);
+  if (p.n_edge == 0) return launch_kind<true>(tm, kf, p.n_full, st);
+  if (p.n_full == 0) return launch_kind<false>(tm, ke, p.n_edge, st);
   // full tiles on the caller's stream, edge tiles concurrently on the side stream
   ForkStream* f = nullptr;
   cast_status s = fork_stream(f);
   if (s != CAST_OK) return s;
   if (cudaEventRecord(f->fork, st) != cudaSuccess || cudaStreamWaitEvent(f->side, f->fork, 0) != cudaSuccess)
     return check_launch("PAR fork");
-  s = launch_kind<T, false>(tm, tm_sw, tm_out, ke, p.n_edge, f->side);
+  s = launch_kind<false>(tm, ke, p.n_edge, f->side);
   if (s != CAST_OK) return s;
-  s = launch_kind<T, true>(tm, tm_sw, tm_out, kf, p.n_full, st);
+  s = launch_kind<true>(tm, kf, p.n_full, st);
   if (cudaEventRecord(f->join, f->side) != cudaSuccess || cudaStreamWaitEvent(st, f->join, 0) != cudaSuccess)
     return check_launch("PAR join");
   return s;
@@ -1173,9 +1640,7 @@ ParPlan par_plan(const cast_par_args& a) {
   // workspace: the chunk records [tile][pair][chunk][kRec] and theta, g [tile][pair][2][kNB]
   p.rec_bytes = align_up((size_t)p.n_tile * (na > 0 ? na : 1) * p.n_chunk * kRec * sizeof(float));
   p.trans_bytes = align_up((size_t)p.n_tile * (na > 0 ? na : 1) * 2 * kNB * sizeof(float));
-  // bf16: the blend matrices of every (tile, target)
-  p.img_bytes = a.dtype == CAST_BF16 ? align_up((size_t)p.n_tile * (p.n_target > 0 ? p.n_target : 1) * kImgBytes) : 0;
-  p.total_bytes = p.n_target > 0 ? p.rec_bytes + p.trans_bytes + p.img_bytes : 0;
+  p.total_bytes = p.n_target > 0 ? p.rec_bytes + p.trans_bytes : 0;
   return p;
 }
 
@@ -1223,8 +1688,6 @@ cast_status launch_par(const cast_par_args& a, void* ws, cudaStream_t st) {
   k.n_chunk = p.n_chunk;
   k.rec = static_cast<float*>(ws);
   k.trans = reinterpret_cast<float*>(static_cast<char*>(ws) + p.rec_bytes);
-  k.img = p.img_bytes ? static_cast<char*>(ws) + p.rec_bytes + p.trans_bytes : nullptr;
-  k.n_target = p.n_target;
   int anchors[CAST_MAX_FRAMES];
   int na = 0;
   for (int f = 0; f < a.F; ++f)
@@ -1263,15 +1726,49 @@ cast_status launch_par(const cast_par_args& a, void* ws, cudaStream_t st) {
   static const FastSrc fast_src = make_fast_src();
   std::copy(fast_src.v, fast_src.v + kNV, k.fast_src);
 
+  if (a.dtype == CAST_BF16) {
+    k.n_full = p.n_full;
+    for (int q = 0; q < 4; ++q) {
+      const int h = (q & 2) ? a.Hg % k.th : k.th, w = (q & 1) ? a.Wg % k.tw : k.tw;
+      if (h > 0 && w > 0) make_slots(h, w, k.bin_slot[q], k.slot_bin[q]);
+    }
+    for (int j = 1; j < na; ++j) {
+      if (k.pair_tbeg[j + 1] > k.pair_tbeg[j]) k.act_pair[k.n_act++] = (unsigned char)j;
+      for (int t = k.pair_tbeg[j]; t < k.pair_tbeg[j + 1]; t += 2, ++k.n_grp) {
+        k.grp_pair[k.n_grp] = (unsigned char)j;
+        k.grp_t0[k.n_grp] = (short)t;
+        k.grp_nt[k.n_grp] = (unsigned char)std::min(2, k.pair_tbeg[j + 1] - t);
+      }
+    }
+    // the range of chunks a unit takes: whole rounds of units over the SMs against what every
+    // unit costs besides its chunks (the reduction of the sums, the first matrices: about as
+    // much as two chunks and one)
+    const int nsm = sm_count();
+    auto split = [&](int64_t units, int extra, int& parts, int& cpp) {
+      int64_t best = -1;
+      for (int q = 1; q <= p.n_chunk; ++q) {
+        const int c = (p.n_chunk + q - 1) / q;
+        if ((p.n_chunk + c - 1) / c != q) continue;   // the same ranges as with fewer parts
+        const int64_t cost = (units * q + nsm - 1) / nsm * (c + extra);
+        if (best < 0 || cost < best) {
+          best = cost;
+          parts = q;
+          cpp = c;
+        }
+      }
+    };
+    split((int64_t)p.n_tile * k.n_act, 2, k.st_parts, k.st_cpp);
+    split((int64_t)p.n_tile * k.n_grp, 1, k.bl_parts, k.bl_cpp);
+    CUtensorMap tm_sw, tm_out;
+    // anchors in boxes of 8 x 8 tokens, outputs in four rows of a tile; other tile sides row by row
+    const bool whole = k.th == 8 && k.tw == 8;
+    if (!make_r_map_sw(&tm_sw, a, k.tw, whole ? 8 : 1) || !make_r_map_sw(&tm_out, a, k.tw, whole ? 4 : 1))
+      return fail(CAST_ERR_CUDA, "PAR: cuTensorMapEncodeTiled failed");
+    return launch_tc(tm_sw, tm_out, k, st);
+  }
   CUtensorMap tm;
   if (!make_r_map(&tm, a, p.chunk)) return fail(CAST_ERR_CUDA, "PAR: cuTensorMapEncodeTiled failed");
-  if (a.dtype == CAST_BF16) {
-    CUtensorMap tm_sw, tm_out;
-    if (!make_r_map_sw(&tm_sw, a, 8, 8) || !make_r_map_sw(&tm_out, a, k.tw, k.th))
-      return fail(CAST_ERR_CUDA, "PAR: cuTensorMapEncodeTiled failed");
-    return launch_typed<__nv_bfloat16>(tm, &tm_sw, &tm_out, k, p, st);
-  }
-  return launch_typed<float>(tm, nullptr, nullptr, k, p, st);
+  return launch_f32(tm, k, p, st);
 }
 
 unsigned int par_error_word(cudaStream_t st, bool clear) {
