@@ -281,6 +281,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     tmem_relinquish();
     tc_fence_before();
   }
+  // the launch behind this one may take SMs as they become free (it waits for this grid's end)
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = bars->tmem_base;

@@ -523,6 +523,7 @@ cast_status cast_block_step(const cast_block_args* a, void* ws, size_t ws_bytes,
       g.c_frame[i] = a->anchors[i];
     }
     g.gelu = false;
+    g.dependent = true;
     if ((s = gemm_anchor_rows(g, st))) return s;
   }
   if (par_plan(p).n_target > 0) {
@@ -631,7 +632,7 @@ cast_status cast_ffn_step(const cast_ffn_args* a, void* ws, size_t ws_bytes, voi
   g2.K = a->D_ff;
   g2.n_anchors = a->n_anchors;
   g2.gelu = false;
-  g2.after_gemm = true;
+  g2.dependent = true;
   for (int i = 0; i < a->n_anchors; ++i) {
     g1.a_frame[i] = a->anchors[i];
     g1.c_frame[i] = i;

@@ -433,7 +433,7 @@ cast_status gemm_anchor_rows(const AnchorGemm& g, cudaStream_t st) {
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
-  cfg.numAttrs = g.after_gemm ? 1 : 0;
+  cfg.numAttrs = g.dependent ? 1 : 0;
   if (cudaLaunchKernelEx(&cfg, k_gemm, ma, mw, k) != cudaSuccess) return check_launch("dense GEMM kernel");
   return check_launch("dense GEMM kernel");
 }

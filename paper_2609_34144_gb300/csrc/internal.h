@@ -143,7 +143,7 @@ struct AnchorGemm {
   int S, N, K, n_anchors;
   int a_frame[CAST_MAX_ANCHORS], c_frame[CAST_MAX_ANCHORS];
   bool gelu;
-  bool after_gemm;   // the launch before on the stream is this kernel's (programmatic dependent)
+  bool dependent;   // programmatic dependent of the launch before it on the stream
 };
 cast_status gemm_anchor_rows(const AnchorGemm& g, cudaStream_t st);
 unsigned int dense_error_word(cudaStream_t st, bool clear);

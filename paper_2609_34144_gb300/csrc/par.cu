@@ -174,7 +174,7 @@ struct ParKArgs {
   // bf16 path (tensor cores)
   int n_full;                            // 8x8 tiles (tiles 0 .. n_full-1; the others follow)
   int n_act, n_grp;                      // pairs with targets; groups of up to two targets of a pair
-  int st_parts, st_cpp, bl_parts, bl_cpp;   // channel-chunk ranges of K_stats_tc / K_blend_tc and chunks in each
+  int st_parts, st_cpp, bl_parts, bl_cpp;   // K_stats_tc / K_blend_tc: channel-chunk ranges and chunks in each
   // per tile shape (bit 0: last column of tiles, truncated; bit 1: last row): where the stored bin
   // b's sums stand in a record (BinSlot), and the bin of each slot (255: none)
   unsigned char bin_slot[4][40], slot_bin[4][34];
@@ -782,6 +782,7 @@ __global__ void __launch_bounds__(kStThreads, 1)
     if (warp == 0 && lane == 0) {
       // -------------------------------------------------------------- anchor producer
       tma_prefetch_desc(&tm);
+      grid_dependency_wait();   // the anchors (what the sums need besides comes after them)
       int n = 0;
       bool ok = true;
       for (int u = blockIdx.x; ok && u < n_units; u += gridDim.x) {
@@ -889,9 +890,9 @@ __global__ void __launch_bounds__(kStThreads, 1)
       };
       for (int c = x.c0; c < x.c1; ++c, ++n) {
         const int buf = n & 1, ch = c * 128 + q4 * 32 + lane;
-        if (WEIGHTED) wc = ch < a.C ? __ldg(a.wch + ch) : 1.f;
         if (!(ok = __all_sync(0xffffffffu, wait(&b_dfull[buf], (uint32_t)(n >> 1) & 1u)))) break;
         tc_fence_after();
+        if (WEIGHTED) wc = ch < a.C ? __ldcg(a.wch + ch) : 1.f;
         // the warpgroup's columns of anchors a and b, then the buffer goes back to its issuer
         uint32_t va[64];
         tmem_ld_x32_async(td0 + (uint32_t)(buf * 256 + wg * kQCols), va);
@@ -1161,7 +1162,7 @@ __global__ void __launch_bounds__(kTbThreads, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = s_tmem;
-  // (only the transport reads what K_stats_tc wrote: its warp waits for that grid)
+  // (the warps that read what earlier launches wrote, 0 and 2, wait for the grid before)
   // unit u -> (tile, target group, chunk range): groups innermost, so that a tile's anchors are
   // read from L2 by the CTAs of neighbouring units
   struct Unit {
@@ -1182,6 +1183,8 @@ __global__ void __launch_bounds__(kTbThreads, 1)
     if (lane == 0) {
       // -------------------------------------------------------------- anchor producer
       tma_prefetch_desc(&tm);
+      // the anchors may come from the launch before the statistics, whose grid waited for it
+      grid_dependency_wait();
       int n = 0;
       bool ok = true;
       for (int u = blockIdx.x; ok && u < n_units; u += gridDim.x) {
@@ -1468,7 +1471,8 @@ bool make_r_map(CUtensorMap* m, const cast_par_args& a, int cc) {
             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// bf16: two launches over every tile, the second a programmatic dependent of the first.
+// bf16: two launches over every tile, each a programmatic dependent of the launch before it on the
+// stream (the statistics kernel sets itself up and builds its operand while that one ends).
 cast_status launch_tc(const CUtensorMap& tm_sw, const CUtensorMap& tm_out, const ParKArgs& k, cudaStream_t st) {
   static std::atomic<uint64_t> attr_done{0};
   if (!once_per_device(attr_done, [] {
@@ -1480,18 +1484,19 @@ cast_status launch_tc(const CUtensorMap& tm_sw, const CUtensorMap& tm_out, const
                    cudaSuccess;
       }))
     return check_launch("PAR kernel attributes");
-  const int nsm = sm_count();
   cudaLaunchAttribute pdl[1];
   pdl[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   pdl[0].val.programmaticStreamSerializationAllowed = 1;
   cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(std::min(k.n_tile * k.n_act * k.st_parts, nsm), 1, 1);
+  cfg.gridDim = dim3(std::min(k.n_tile * k.n_act * k.st_parts, sm_count()), 1, 1);
   cfg.blockDim = dim3(kStThreads, 1, 1);
   cfg.dynamicSmemBytes = kStSmem;
   cfg.stream = st;
+  cfg.attrs = pdl;
+  cfg.numAttrs = 1;
   if (cudaLaunchKernelEx(&cfg, k.wch ? k_par_stats_tc<true> : k_par_stats_tc<false>, tm_sw, k) != cudaSuccess) return check_launch("PAR statistics kernel");
   cudaLaunchConfig_t bc{};
-  bc.gridDim = dim3(std::min(k.n_tile * k.n_grp * k.bl_parts, nsm), 1, 1);
+  bc.gridDim = dim3(std::min(k.n_tile * k.n_grp * k.bl_parts, sm_count()), 1, 1);
   bc.blockDim = dim3(kTbThreads, 1, 1);
   bc.dynamicSmemBytes = kTbSmem;
   bc.stream = st;
@@ -1740,16 +1745,20 @@ cast_status launch_par(const cast_par_args& a, void* ws, cudaStream_t st) {
         k.grp_nt[k.n_grp] = (unsigned char)std::min(2, k.pair_tbeg[j + 1] - t);
       }
     }
-    // the range of chunks a unit takes: whole rounds of units over the SMs against what every
-    // unit costs besides its chunks (the reduction of the sums, the first matrices: about as
-    // much as two chunks and one)
+    // The range of chunks a unit takes.  CTAs stride the units (contiguous ranges of units per CTA
+    // lose the anchors' reuse in L2: HY-World-shaped 109 -> 123 us); a unit takes its chunks
+    // and what does not overlap with the neighbours' work, and the first one `start` more (all in
+    // chunks): the statistics' reduction takes about one chunk (1,100 cycles) and their start four
+    // (6,000 cycles until the first products: the DFT operand); a unit of the blend takes at least
+    // six (transport and matrices of the next one, 8,000 cycles) and the first one eight.
     const int nsm = sm_count();
-    auto split = [&](int64_t units, int extra, int& parts, int& cpp) {
+    auto split = [&](int64_t units, int extra, int least, int start, int& parts, int& cpp) {
       int64_t best = -1;
       for (int q = 1; q <= p.n_chunk; ++q) {
         const int c = (p.n_chunk + q - 1) / q;
         if ((p.n_chunk + c - 1) / c != q) continue;   // the same ranges as with fewer parts
-        const int64_t cost = (units * q + nsm - 1) / nsm * (c + extra);
+        const int64_t n = (units * q + nsm - 1) / nsm;
+        const int64_t cost = start + (n - 1) * std::max(c + extra, least) + c + extra;
         if (best < 0 || cost < best) {
           best = cost;
           parts = q;
@@ -1757,8 +1766,8 @@ cast_status launch_par(const cast_par_args& a, void* ws, cudaStream_t st) {
         }
       }
     };
-    split((int64_t)p.n_tile * k.n_act, 2, k.st_parts, k.st_cpp);
-    split((int64_t)p.n_tile * k.n_grp, 1, k.bl_parts, k.bl_cpp);
+    split((int64_t)p.n_tile * k.n_act, 1, 0, 4, k.st_parts, k.st_cpp);
+    split((int64_t)p.n_tile * k.n_grp, 0, 6, 8, k.bl_parts, k.bl_cpp);
     CUtensorMap tm_sw, tm_out;
     // anchors in boxes of 8 x 8 tokens, outputs in four rows of a tile; other tile sides row by row
     const bool whole = k.th == 8 && k.tw == 8;
