@@ -571,13 +571,12 @@ def _captured_traffic():
 
 # ------------------------------------------------------------------------------ CPU oracle
 def launches_per_step(wl):
-    """Library kernels one block step launches: pooling (anchor frames, history blocks) and
-    the per-head routing kernel, attention, and PAR (statistics, transport and blend passes
-    for the full 8x8 tiles and for the truncated edge tiles when the grid has both)."""
+    """Library kernels one block step launches: pooling (history blocks, anchor frames) and the
+    per-head routing kernel, attention, and PAR (bf16: statistics and blend, both over every tile;
+    f32: statistics, transport and blend of the full 8x8 tiles and of the truncated edge tiles)."""
     hg, wg = wl.grid
-    full = (hg // 8) * (wg // 8) > 0
-    edge = hg % 8 != 0 or wg % 8 != 0
-    return 3 + 1 + 3 * (int(full) + int(edge))
+    kinds = int((hg // 8) * (wg // 8) > 0) + int(hg % 8 != 0 or wg % 8 != 0)
+    return 3 + 1 + (2 if wl.dtype == "bf16" else 3 * kinds)
 
 
 # One bounded sample of the block step, the same for the `cpu_baseline` leg and for `--impl
