@@ -1063,73 +1063,89 @@ __device__ __forceinline__ float masked(const float* key, const uint8_t* cm, int
   return (cm && !cm[p]) ? -INFINITY : key[p];
 }
 
+// f(m, order key) for the blocks of one row that this thread owns (m = thread + 256 k, ascending):
+// the first kKeyRegs keys come from kreg, the others are formed from key[] and cm[] again.
+constexpr int kKeyRegs = 4;
+template <typename F>
+__device__ __forceinline__ void each_key(const unsigned long long (&kreg)[kKeyRegs], const float* key,
+                                         const uint8_t* cm, int M, F&& f) {
+#pragma unroll
+  for (int k = 0; k < kKeyRegs; ++k) {
+    const int m = threadIdx.x + k * kWideThreads;
+    if (m < M) f(m, kreg[k]);
+  }
+  for (int m = threadIdx.x + kKeyRegs * kWideThreads; m < M; m += kWideThreads)
+    f(m, order_key(masked(key, cm, m), m));
+}
+
 // Radix select of the TopK threshold of one row key[0..M) (entries with cm[m] == 0 count as
 // -inf; 0 < K < M): returns the order key t such that exactly K keys of the row have
-// order_key >= t.  Rounds of 10-bit digits from the top of the 46-bit key; a round whose
-// chosen digit holds exactly the remaining count ends the select (its lower bits are then
-// left zero).  hist holds two 1024-bin buffers, zero on entry and zero again on return; each
-// round's buffer is cleared during the round after it.  Every thread of the CTA calls this.
-__device__ unsigned long long topk_threshold(const float* key, const uint8_t* cm, int M, int K,
-                                             unsigned* hist2, unsigned long long* sel) {
-  const int tid = threadIdx.x, lane = tid & 31;
+// order_key >= t, and this thread's own keys in kreg.  Rounds of 10-bit digits from the top of the
+// 46-bit key; a round whose chosen digit holds exactly the remaining count ends the select (its
+// lower bits are then left zero), usually the second.  hist: 1024 bins, zero on entry and on
+// return; wsum: a word per warp.  Every thread of the CTA calls this, with key[] of its own blocks
+// written by itself.
+// Bound by its chain of dependent steps, so every warp takes part in each (four bins per thread,
+// cleared as they are read), and the keys are formed once: 4,090 cycles a select at 448 blocks with
+// one warp adding up all bins, two buffers cleared in turn and the keys formed in each round; the
+// routing call with 448 blocks, 4 anchors and 2 passes (12 selects) took 96 us then, 87 us now.
+__device__ unsigned long long topk_threshold(const float* key, const uint8_t* cm, int M, int K, unsigned* hist,
+                                             unsigned* wsum, unsigned long long* sel,
+                                             unsigned long long (&kreg)[kKeyRegs]) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+#pragma unroll
+  for (int k = 0; k < kKeyRegs; ++k) {
+    const int m = tid + k * kWideThreads;
+    kreg[k] = m < M ? order_key(masked(key, cm, m), m) : 0ull;
+  }
   unsigned long long pre = 0ull;
   int krem = K;
-  int round = 0;
-  for (int shift = 36;; shift = shift >= 10 ? shift - 10 : 0, ++round) {
+  for (int shift = 36;; shift = shift >= 10 ? shift - 10 : 0) {
     const int width = shift == 0 ? 6 : 10;   // bits 45..36, 35..26, 25..16, 15..6, 5..0
-    // (the last round's 6-bit digit uses bins 0..63 of the same 1024)
-    unsigned* hist = hist2 + (round & 1) * kRadixBins;
-    if (round > 0)   // the previous round's buffer is free again (read before the last barrier)
-      for (int e = tid; e < kRadixBins; e += kWideThreads) hist2[((round - 1) & 1) * kRadixBins + e] = 0u;
+    // (the last round's digit keeps four known bits above its six)
     const unsigned long long hi = ~0ull << (shift + width);
-    for (int m = tid; m < M; m += kWideThreads) {
-      const unsigned long long c = order_key(cm && !cm[m] ? -INFINITY : key[m], m);
+    each_key(kreg, key, cm, M, [&](int, unsigned long long c) {
       if ((c & hi) == pre) atomicAdd(&hist[(int)((c >> shift) & (unsigned long long)(kRadixBins - 1))], 1u);
-    }
+    });
     __syncthreads();
-    if (tid < 32) {
-      // the digit where the count from the top reaches krem: lane l first sums the 32 bins
-      // 1023-32l .. 992-32l (rotated so the lanes hit different banks), a warp scan picks the
-      // chunk, then the warp scans that chunk's bins
-      unsigned part = 0;
-#pragma unroll 8
-      for (int t = 0; t < 32; ++t) part += hist[kRadixBins - 1 - 32 * lane - ((t + lane) & 31)];
-      unsigned inc = part;
+    // the digit where the count from the top reaches krem: thread t takes the bins 1023 - 4 t ..
+    // 1020 - 4 t, a warp scan and the totals of the warps above give the count before them
+    uint4* mine = reinterpret_cast<uint4*>(hist + kRadixBins - 4 - 4 * tid);
+    const uint4 v = *mine;
+    *mine = make_uint4(0u, 0u, 0u, 0u);
+    const unsigned own = v.x + v.y + v.z + v.w;
+    unsigned inc = own;
 #pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const unsigned w = __shfl_up_sync(0xffffffffu, inc, o);
-        if (lane >= o) inc += w;
-      }
-      const int l = __ffs(__ballot_sync(0xffffffffu, inc >= (unsigned)krem)) - 1;
-      const unsigned carry = __shfl_sync(0xffffffffu, inc - part, l);
-      const int b = kRadixBins - 1 - 32 * l - lane;
-      const unsigned v = hist[b];
-      unsigned inc2 = v;
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned w = __shfl_up_sync(0xffffffffu, inc, o);
+      if (lane >= o) inc += w;
+    }
+    if (lane == 31) wsum[warp] = inc;
+    __syncthreads();
+    unsigned before = inc - own;
 #pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const unsigned w = __shfl_up_sync(0xffffffffu, inc2, o);
-        if (lane >= o) inc2 += w;
-      }
-      const int j = __ffs(__ballot_sync(0xffffffffu, carry + inc2 >= (unsigned)krem)) - 1;
-      if (lane == j) {
-        const unsigned before = carry + inc2 - v;
-        sel[0] = pre | ((unsigned long long)b << shift);
-        sel[1] = (unsigned long long)(krem - (int)before);
-        sel[2] = (v == (unsigned)krem - before || shift == 0) ? 1ull : 0ull;
-      }
+    for (int w = 0; w < kWideWarps; ++w) before += w < warp ? wsum[w] : 0u;
+    if (before < (unsigned)krem && before + own >= (unsigned)krem) {
+      const unsigned n[4] = {v.w, v.z, v.y, v.x};
+      int d = 0;
+#pragma unroll
+      for (int e = 0; e < 3; ++e)
+        if (d == e && before + n[e] < (unsigned)krem) {
+          before += n[e];
+          d = e + 1;
+        }
+      const unsigned left = (unsigned)krem - before, at = d == 0 ? n[0] : d == 1 ? n[1] : d == 2 ? n[2] : n[3];
+      sel[0] = pre | ((unsigned long long)(kRadixBins - 1 - 4 * tid - d) << shift);
+      sel[1] = (unsigned long long)left;
+      sel[2] = (at == left || shift == 0) ? 1ull : 0ull;
     }
     __syncthreads();
     pre = sel[0];
     krem = (int)sel[1];
-    const bool done = sel[2] != 0ull;
-    if (done) {
-      // clear this round's buffer before leaving (the other one is already zero)
-      for (int e = tid; e < kRadixBins; e += kWideThreads) hist[e] = 0u;
-      __syncthreads();
-      return pre;
-    }
+    if (sel[2] != 0ull) return pre;
   }
 }
+static_assert(4 * kWideThreads == kRadixBins, "four bins per thread");
 
 // Deterministic CTA-wide sum (warp sums added in warp order); every thread gets the total.
 // red2 holds two slot sets used alternately (`slot` flips between calls), so a call never
@@ -1390,7 +1406,9 @@ __global__ void __launch_bounds__(kWideThreads) k_head_wide(const __grid_constan
       if (lane == 0 && n != a.Mc) atomicExch(&g_route_error, 1u);
     }
   }
-  for (int e = tid; e < 2 * kRadixBins; e += kWideThreads) hist[e] = 0u;
+  unsigned* wsum = reinterpret_cast<unsigned*>(red2 + 32);   // behind the two sets of block_sum
+  unsigned long long kreg[kKeyRegs];
+  for (int e = tid; e < kRadixBins; e += kWideThreads) hist[e] = 0u;
   int slot = 0;
   __syncthreads();
   // initial masks: TopK of each anchor's key (Eq. topk), within C_i
@@ -1399,9 +1417,8 @@ __global__ void __launch_bounds__(kWideThreads) k_head_wide(const __grid_constan
   } else {
     for (int i = 0; i < na; ++i) {
       const uint8_t* cmi = cm ? cm + i * M : nullptr;
-      const unsigned long long t = topk_threshold(u + i * M, cmi, M, K, hist, sel);
-      for (int m = tid; m < M; m += kWideThreads)
-        x[i * M + m] = order_key(masked(u + i * M, cmi, m), m) >= t ? 1.f : 0.f;
+      const unsigned long long t = topk_threshold(u + i * M, cmi, M, K, hist, wsum, sel, kreg);
+      each_key(kreg, u + i * M, cmi, M, [&](int m, unsigned long long c) { x[i * M + m] = c >= t ? 1.f : 0.f; });
     }
   }
   __syncthreads();
@@ -1458,20 +1475,18 @@ __global__ void __launch_bounds__(kWideThreads) k_head_wide(const __grid_constan
           }
           G[m] = lam_anc * ui + lam_rec * rec;
         }
-        __syncthreads();
         // best response TopK(G) within C_i and its gain sum_m G_m (x_new - x_i); J is affine in
         // x_i, so the accepted step lowers J by exactly that gain
         const uint8_t* cmi = cm ? cm + i * M : nullptr;
-        const unsigned long long thr = topk_threshold(G, cmi, M, K, hist, sel);
+        const unsigned long long thr = topk_threshold(G, cmi, M, K, hist, wsum, sel, kreg);
         float gl = 0.f;
-        for (int m = tid; m < M; m += kWideThreads) {
-          const float nx = order_key(masked(G, cmi, m), m) >= thr ? 1.f : 0.f;
+        each_key(kreg, G, cmi, M, [&](int m, unsigned long long c) {
+          const float nx = c >= thr ? 1.f : 0.f;
           gl += G[m] * (nx - x[i * M + m]);
-        }
+        });
         const float gain = block_sum(gl, red2, slot);
         if (gain > a.tol * fmaxf(J, 1e-8f)) {   // uniform across the CTA
-          for (int m = tid; m < M; m += kWideThreads)
-            x[i * M + m] = order_key(masked(G, cmi, m), m) >= thr ? 1.f : 0.f;
+          each_key(kreg, G, cmi, M, [&](int m, unsigned long long c) { x[i * M + m] = c >= thr ? 1.f : 0.f; });
           J -= gain;
           changed = true;
         }
@@ -1485,6 +1500,7 @@ __global__ void __launch_bounds__(kWideThreads) k_head_wide(const __grid_constan
   for (int i = warp; i < na; i += kWideWarps) {
     int base = 0;
     int32_t* out = a.idx + ((int64_t)i * a.H + h) * K;
+#pragma unroll 4
     for (int mb = 0; mb < M; mb += 32) {
       const int m = mb + lane;
       const bool on = m < M && x[i * M + m] != 0.f;
