@@ -145,6 +145,23 @@ __device__ __forceinline__ void load_vec_smem(const uint8_t* p, float (&x)[16 / 
   }
 }
 
+// r / w of a row r of a (1, 8, 8) block with runs of w tokens as (r run_reciprocal(w)) >> 16
+__host__ __device__ constexpr uint32_t run_reciprocal(int w) { return (65535u + w) / w; }
+constexpr bool run_quotients_exact() {
+  for (int w = 1; w <= 8; ++w)
+    for (int r = 0; r < 64; ++r)
+      if (((r * run_reciprocal(w)) >> 16) != (uint32_t)(r / w)) return false;
+  return true;
+}
+static_assert(run_quotients_exact(), "rows of a block");
+
+// Registers per thread.  SPATIAL segments are short (64 rows), so most of a CTA's life is the latency
+// of its first loads and its last sums: three CTAs of 384 threads per SM (56 registers, 147 KB of
+// loads in flight) instead of two (64 registers, with a division and a 64-bit product per row address)
+// took the history pooling of 448 blocks x 3 KB rows from 38 to 30 us, the routing call from 87 to
+// 81 us.  The long segments of the other forms already fill the SMs.
+constexpr int pool_regs(size_t elt, bool spatial) { return spatial ? 56 : elt == 2 ? 64 : 40; }
+
 // grid (nsplit, n_seg), cluster (nsplit, 1, 1), cgs * lanes_r threads.  Dynamic smem:
 // colsum[D] and (lanes_r - 1) rows of per-lane sums (then, BULK, the copy ring).  SPATIAL: the
 // history segments are (1, 8, 8) blocks of frames [frames][Hg][Wg] (hv runs of wv consecutive
@@ -152,7 +169,7 @@ __device__ __forceinline__ void load_vec_smem(const uint8_t* p, float (&x)[16 / 
 // one 16-byte column group per thread): the CTA's rows arrive through a ring of bulk copies of
 // bulk_rows rows each, so that two CTAs keep about 190 KB of loads in flight per SM.
 template <typename T, bool SPATIAL, bool BULK>
-__global__ void __launch_bounds__(kPoolMaxThreads) k_pool(const __grid_constant__ PoolArgs a) {
+__global__ void __maxnreg__(pool_regs(sizeof(T), SPATIAL)) k_pool(const __grid_constant__ PoolArgs a) {
   constexpr int VEC = 16 / sizeof(T);
   extern __shared__ float colsum[];
   launch_dependents();
@@ -160,8 +177,9 @@ __global__ void __launch_bounds__(kPoolMaxThreads) k_pool(const __grid_constant_
   const char* base;
   int64_t rs;
   int nrows;
-  int run = 1 << 30;      // SPATIAL: tokens per run (wv) and rows between runs (Wg)
-  int64_t run_stride = 0;
+  // SPATIAL: row r is token r % wv of run r / wv, r + (r / wv) run_skip tokens from the first
+  uint32_t run_inv = 0;
+  int run_skip = 0;
   float* out;
   if (seg < a.n_anchors) {
     base = a.q + (int64_t)a.anchors[seg] * a.S * a.q_row_stride * a.elt;
@@ -181,8 +199,8 @@ __global__ void __launch_bounds__(kPoolMaxThreads) k_pool(const __grid_constant_
       const int hv = min(8, a.Hg - 8 * by), wv = min(8, a.Wg - 8 * bx);
       base = src + (((int64_t)f * a.Hg + 8 * by) * a.Wg + 8 * bx) * rs * a.elt;
       nrows = hv * wv;
-      run = wv;
-      run_stride = a.Wg;
+      run_inv = run_reciprocal(wv);
+      run_skip = a.Wg - wv;
     } else {
       base = src + (int64_t)m * a.B_v * rs * a.elt;
       nrows = a.B_v;
@@ -258,12 +276,9 @@ __global__ void __launch_bounds__(kPoolMaxThreads) k_pool(const __grid_constant_
 #pragma unroll
     for (int k = 0; k < VEC; ++k) acc[k] = 0.f;
     if (SPATIAL && trl < lanes_r) {
-      // row r of the segment: run r / wv, token r % wv of that run
       const char* pc = base + (int64_t)cg * VEC * a.elt;
-      auto rowp = [&](int r) {
-        const int y = r / run;
-        return pc + ((int64_t)y * run_stride + (r - y * run)) * rs * a.elt;
-      };
+      const int64_t row_bytes = rs * a.elt;
+      auto rowp = [&](int r) { return pc + (int64_t)(r + (int)((r * run_inv) >> 16) * run_skip) * row_bytes; };
       int r = r0 + trl;
       for (; r + (kPoolUnroll - 1) * lanes_r < r1; r += kPoolUnroll * lanes_r) {
         float x[kPoolUnroll][VEC];
