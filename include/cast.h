@@ -104,7 +104,8 @@ typedef struct {
   int64_t hist_row_stride;
   int32_t M, B_v;
   /* Gram matrices G_h = P_h^T P_h of the output-projection head slices P = W_O^(h),
-     device f32 [H, d, d]; NULL means P = I (u = ||delta||^2) */
+     device f32 [H, d, d] at any 4-byte boundary (16 bytes are read faster); NULL means P = I
+     (u = ||delta||^2) */
   const float* gram;
   int32_t K;                      /* budget K_KV; K_eff = min(K, M) blocks are kept */
   float eps;                      /* stabiliser of Eq. (omission); 1e-8 by default */
@@ -142,9 +143,9 @@ typedef struct {
  * With CAST_HIST_FRAMES a block's means run over its own tokens (64, or fewer at the grid
  * edge).
  * Errors: INVALID_ARG for NULL required pointers, n_anchors < 1 or > CAST_MAX_ANCHORS,
- * anchors not ascending / out of range, K < 0, M < 0, B_v < 1 with M > 0, bad strides,
- * an unknown hist.kind, or CAST_HIST_FRAMES with a non-positive grid, M different from its
- * block count or B_v != 64,
+ * anchors not ascending / out of range, K < 0, M < 0, B_v < 1 with M > 0, bad strides, a gram
+ * that is read and lies off a 4-byte boundary, an unknown hist.kind, or CAST_HIST_FRAMES with a
+ * non-positive grid, M different from its block count or B_v != 64,
  * a workspace smaller than cast_route_workspace_size(), refinement with a negative weight or
  * tolerance or outside CAST_ROUTE_OMISSION, candidates with M_c outside K_eff..M; a candidate
  * index outside [0, M) or repeated within a set makes the kernel record an error that

@@ -169,6 +169,8 @@ cast_status validate_route(const cast_route_args* a) {
   for (const float* p : {a->qbar, a->kbar, a->vbar})
     if (reinterpret_cast<uintptr_t>(p) % 16)
       return fail(CAST_ERR_INVALID_ARG, "%s: qbar/kbar/vbar must be 16-byte aligned", who);
+  if (a->M > 0 && a->mode == CAST_ROUTE_OMISSION && reinterpret_cast<uintptr_t>(a->gram) % 4)
+    return fail(CAST_ERR_INVALID_ARG, "%s: gram misaligned", who);
   if (!(a->eps >= 0.f)) return fail(CAST_ERR_INVALID_ARG, "%s: eps must be >= 0", who);
   if (a->refine_passes < 0) return fail(CAST_ERR_INVALID_ARG, "%s: refine_passes < 0", who);
   if (a->refine_passes > 0) {

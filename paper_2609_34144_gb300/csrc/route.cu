@@ -421,6 +421,8 @@ __device__ __forceinline__ float warp_total(float v) { return warp_sum(v); }
 // row, cost 613 us for 12 heads of 4 anchors x 16 blocks (2,290 us for the projected
 // Matrix-Game-shaped block step).  y_r sums over c in order and the rows of a lane in order, as
 // before: the scores are the same bits.
+// G may start anywhere a float can (a matrix within a packed buffer of weights): off a 16-byte
+// boundary its columns are read one float at a time.
 constexpr int kGramPairs = 8, kGramCols = 32;
 __host__ __device__ constexpr size_t gram_stage_bytes(int d) { return (size_t)d * (kGramCols + 1) * sizeof(float); }
 
@@ -430,6 +432,7 @@ __device__ void gram_scores(const float* __restrict__ G, const float* ob, const 
   constexpr int R = HD / 32, kPer = HD * kGramCols / 4 / kHeadThreads;   // float4 loads per thread and stage
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int n_pairs = na * nm;
+  const bool aligned = (reinterpret_cast<uintptr_t>(G) & 15u) == 0;
   constexpr int kBatch = kHeadWarps * kGramPairs;
   for (int b0 = 0; b0 < n_pairs; b0 += kBatch) {
     const float *op[kGramPairs], *vp[kGramPairs];
@@ -444,10 +447,19 @@ __device__ void gram_scores(const float* __restrict__ G, const float* ob, const 
     }
     for (int c0 = 0; c0 < HD; c0 += kGramCols) {
       float4 g4[kPer];
+      if (aligned) {
 #pragma unroll
-      for (int t = 0; t < kPer; ++t) {
-        const int e = tid + t * kHeadThreads;
-        g4[t] = __ldg(reinterpret_cast<const float4*>(G + (int64_t)(e >> 3) * HD + c0) + (e & 7));
+        for (int t = 0; t < kPer; ++t) {
+          const int e = tid + t * kHeadThreads;
+          g4[t] = __ldg(reinterpret_cast<const float4*>(G + (int64_t)(e >> 3) * HD + c0) + (e & 7));
+        }
+      } else {
+#pragma unroll
+        for (int t = 0; t < kPer; ++t) {
+          const int e = tid + t * kHeadThreads;
+          const float* p = G + (int64_t)(e >> 3) * HD + c0 + (e & 7) * 4;
+          g4[t] = make_float4(__ldg(p), __ldg(p + 1), __ldg(p + 2), __ldg(p + 3));
+        }
       }
       __syncthreads();   // the stage before has been read
 #pragma unroll
