@@ -390,12 +390,11 @@ __global__ void __launch_bounds__(kThreads, 1)
     auto wait2 = [&](uint64_t* b0, int ph0, uint64_t* b1, int ph1) -> bool {
       uint64_t* const b = lane < 16 ? b0 : b1;
       const uint32_t par = (uint32_t)(lane < 16 ? ph0 : ph1) & 1u;
-      if (__all_sync(0xffffffffu, mbar_try_wait(b, par))) return true;
       uint64_t t0 = 0;
-      for (uint32_t it = 1;; ++it) {
-        if (__all_sync(0xffffffffu, mbar_try_wait(b, par))) return true;
+      for (uint32_t it = 1; !__all_sync(0xffffffffu, mbar_try_wait(b, par)); ++it)
         if (it % kWaitTries == 0 && expired(t0)) return false;
-      }
+      __syncwarp();   // a vote orders no memory: what the other half waited for, the issuing lane sees after this
+      return true;
     };
     auto wait = [&](uint64_t* bar, int phase) -> bool { return wait2(bar, phase, bar, phase); };
     const bool lead = elect_one();   // the same lane issues and commits everything

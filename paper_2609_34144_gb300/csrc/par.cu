@@ -826,6 +826,7 @@ __global__ void __launch_bounds__(kStThreads, 1)
           const bool w = lane < 16 ? wait(&b_full[s], (uint32_t)(n / kStStages) & 1u)
                                    : n < 2 || wait(&b_dempty[buf], (uint32_t)((n >> 1) - 1) & 1u);
           if (!(ok = __all_sync(0xffffffffu, w))) break;
+          __syncwarp();   // (a vote orders no memory) what the other half waited for, the lead sees after this
           tc_fence_after();
           if (lead) {
             const uint64_t da = dx + (uint64_t)(2 * s * (kStTile >> 4));
@@ -1356,6 +1357,7 @@ __global__ void __launch_bounds__(kTbThreads, 1)
         const bool w = lane < 16 ? wait(&b_xfull[s], (uint32_t)(n / kTbStages) & 1u)
                                  : n < 2 || wait(&b_dempty[buf], (uint32_t)((n >> 1) - 1) & 1u);
         if (!(ok = __all_sync(0xffffffffu, w))) break;
+        __syncwarp();   // (a vote orders no memory) what the other half waited for, the lead sees after this
         tc_fence_after();
         if (lead) {
           const uint64_t db = dx + (uint64_t)(s * (kTbStage >> 4));
