@@ -724,7 +724,8 @@ __global__ void __launch_bounds__(kStThreads, 1)
   uint8_t* s_x = dsm;
   uint8_t* s_img = dsm + kStStages * 2 * kStTile;
   float* s_red = reinterpret_cast<float*>(s_img + 3 * kStPiece);   // [2][16 warps][32]
-  __shared__ __align__(8) uint64_t b_full[kStStages], b_empty[kStStages], b_dfull[2], b_dempty[2], b_img;
+  __shared__ __align__(8) uint64_t b_full[kStStages], b_empty[kStStages], b_dfull[2], b_dempty[2], b_img,
+      b_seen;
   __shared__ uint32_t s_tmem;
   __shared__ volatile int s_abort;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -748,6 +749,7 @@ __global__ void __launch_bounds__(kStThreads, 1)
       mbar_init(&b_dempty[b], kStSumWarps);
     }
     mbar_init(&b_img, 1);
+    mbar_init(&b_seen, 2);   // both issuers
     fence_barrier_init();
     s_abort = 0;
   }
@@ -817,6 +819,7 @@ __global__ void __launch_bounds__(kStThreads, 1)
         if (g.h * 16 + g.w != shape) {
           shape = g.h * 16 + g.w;
           if (!(ok = __all_sync(0xffffffffu, wait(&b_img, (uint32_t)builds++ & 1u)))) break;
+          if (lane == 0) mbar_arrive(&b_seen);
         }
         const bool pieces = !(g.h == 8 && g.w == 8);
         for (int c = x.c0; c < x.c1; ++c, ++n) {
@@ -860,7 +863,7 @@ __global__ void __launch_bounds__(kStThreads, 1)
     const int wg = (warp >> 2) - 1, q4 = warp & 3, ctid = tid - 128;
     const uint32_t td0 = tmem + ((uint32_t)(q4 * 32) << 16);
     constexpr float kR = 0.70710678118654752f;
-    int n = 0, shape = -1, flip = 0;
+    int n = 0, shape = -1, builds = 0, flip = 0;
     bool ok = true;
     for (int u = blockIdx.x; u < n_units; u += gridDim.x, flip ^= 1) {
       const Unit x = unit_of(u);
@@ -871,7 +874,10 @@ __global__ void __launch_bounds__(kStThreads, 1)
         build_dft_operand(a, g, s_img, ctid);
         fence_proxy_async_smem();
         stats_sync();
-        if (ctid == 0) mbar_arrive(&b_img);
+        // an issuer without a chunk since then may not have seen the operand before this one: its
+        // barrier must not run a second phase ahead of it
+        if (ctid == 0 && (builds == 0 || wait(&b_seen, (uint32_t)(builds - 1) & 1u))) mbar_arrive(&b_img);
+        ++builds;
       }
       // Re Z, Im Z, W of the complex bins; of the last warpgroup, Z of the real bins in zr[6],
       // zr[7], zi[6], zi[7] and W in wv[6], wv[7], ex[0], ex[1]
