@@ -863,37 +863,41 @@ __global__ void __launch_bounds__(kStThreads, 1)
     const int wg = (warp >> 2) - 1, q4 = warp & 3, ctid = tid - 128;
     const uint32_t td0 = tmem + ((uint32_t)(q4 * 32) << 16);
     constexpr float kR = 0.70710678118654752f;
-    int n = 0, shape = -1, builds = 0, flip = 0;
+    int n = 0, shape = 0, flip = 0;   // shape: operands built so far << 8 | sides of the last one
     bool ok = true;
     for (int u = blockIdx.x; u < n_units; u += gridDim.x, flip ^= 1) {
       const Unit x = unit_of(u);
       const TileGeom g = any_tile(a, x.tile);
-      if (g.h * 16 + g.w != shape) {
+      if (g.h * 16 + g.w != (shape & 255)) {
         // every UMMA that read the operand has completed: its chunk has been waited for
-        shape = g.h * 16 + g.w;
+        const int builds = shape >> 8;
+        shape = (builds + 1) << 8 | (g.h * 16 + g.w);
         build_dft_operand(a, g, s_img, ctid);
         fence_proxy_async_smem();
         stats_sync();
         // an issuer without a chunk since then may not have seen the operand before this one: its
         // barrier must not run a second phase ahead of it
         if (ctid == 0 && (builds == 0 || wait(&b_seen, (uint32_t)(builds - 1) & 1u))) mbar_arrive(&b_img);
-        ++builds;
       }
       // Re Z, Im Z, W of the complex bins; of the last warpgroup, Z of the real bins in zr[6],
       // zr[7], zi[6], zi[7] and W in wv[6], wv[7], ex[0], ex[1]
       float zr[kQCpx], zi[kQCpx], wv[kQCpx], ex[2] = {0.f, 0.f};
 #pragma unroll
       for (int c = 0; c < kQCpx; ++c) zr[c] = zi[c] = wv[c] = 0.f;
-      // one complex bin; the weight goes on anchor a (w >= 0, so |w F_a| = w |F_a|)
+      // one complex bin; the weight comes last, so that no square of it is formed (w^2 leaves the range
+      // of a float long before w |F_a| |F_b| does)
       float wc = 1.f;
       auto add = [&](int s, float ra, float ia, float rb, float ib) {
+        const float aw = sqrt_approx(fmaf(ra, ra, ia * ia) * fmaf(rb, rb, ib * ib));
         if (WEIGHTED) {
-          ra *= wc;
-          ia *= wc;
+          zr[s] = fmaf(wc, fmaf(rb, ra, ib * ia), zr[s]);
+          zi[s] = fmaf(wc, fmaf(ib, ra, -rb * ia), zi[s]);
+          wv[s] = fmaf(wc, aw, wv[s]);
+        } else {
+          zr[s] = fmaf(rb, ra, fmaf(ib, ia, zr[s]));
+          zi[s] = fmaf(ib, ra, fmaf(-rb, ia, zi[s]));
+          wv[s] += aw;
         }
-        zr[s] = fmaf(rb, ra, fmaf(ib, ia, zr[s]));
-        zi[s] = fmaf(ib, ra, fmaf(-rb, ia, zi[s]));
-        wv[s] += sqrt_approx(fmaf(ra, ra, ia * ia) * fmaf(rb, rb, ib * ib));
       };
       for (int c = x.c0; c < x.c1; ++c, ++n) {
         const int buf = n & 1, ch = c * 128 + q4 * 32 + lane;
@@ -919,7 +923,7 @@ __global__ void __launch_bounds__(kStThreads, 1)
           add(kQOdd, fa[0], fa[1], fb[0], fb[1]);
           add(kQOdd + 1, fa[2], fa[3], fb[2], fb[3]);
         } else {
-          const float z0 = wc * fa[0] * fb[0], z1 = wc * fa[1] * fb[1], z2 = wc * fa[2] * fb[2], z3 = wc * fa[3] * fb[3];
+          const float z0 = wc * (fa[0] * fb[0]), z1 = wc * (fa[1] * fb[1]), z2 = wc * (fa[2] * fb[2]), z3 = wc * (fa[3] * fb[3]);
           zr[kQOdd] += z0;
           zr[kQOdd + 1] += z1;
           zi[kQOdd] += z2;
