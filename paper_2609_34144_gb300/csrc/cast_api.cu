@@ -446,7 +446,7 @@ cast_status cast_par_reconstruct(const cast_par_args* a, void* ws, size_t ws_byt
                 p.total_bytes);
   if (reinterpret_cast<uintptr_t>(ws) % kWsAlign)
     return fail(CAST_ERR_INVALID_ARG, "cast_par_reconstruct: workspace not 256-byte aligned");
-  return launch_par(*a, ws, static_cast<cudaStream_t>(stream));
+  return launch_par(*a, ws, static_cast<cudaStream_t>(stream), false);
 }
 
 size_t cast_block_workspace_size(const cast_block_args* a) {
@@ -529,7 +529,7 @@ cast_status cast_block_step(const cast_block_args* a, void* ws, size_t ws_bytes,
     if ((s = gemm_anchor_rows(g, st))) return s;
   }
   if (par_plan(p).n_target > 0) {
-    if ((s = launch_par(p, w + bp.route_bytes + bp.idx_bytes + bp.attn_bytes, st))) return s;
+    if ((s = launch_par(p, w + bp.route_bytes + bp.idx_bytes + bp.attn_bytes, st, true))) return s;
   }
   if (a->x) {
     const size_t n = (size_t)a->n_frames * a->Hg * a->Wg * a->H * a->d;
@@ -643,7 +643,7 @@ cast_status cast_ffn_step(const cast_ffn_args* a, void* ws, size_t ws_bytes, voi
   }
   if ((s = gemm_anchor_rows(g1, st))) return s;
   if ((s = gemm_anchor_rows(g2, st))) return s;
-  if (par_plan(p).n_target > 0) return launch_par(p, pws, st);
+  if (par_plan(p).n_target > 0) return launch_par(p, pws, st, true);
   return CAST_OK;
 }
 

@@ -121,7 +121,8 @@ struct ParPlan {
   size_t rec_bytes, trans_bytes, total_bytes;   // workspace: chunk records, theta and g
 };
 ParPlan par_plan(const cast_par_args& a);
-cast_status launch_par(const cast_par_args& a, void* ws, cudaStream_t st);
+// after_own: the launch before on the stream is a kernel of this library (attention or GEMM)
+cast_status launch_par(const cast_par_args& a, void* ws, cudaStream_t st, bool after_own);
 unsigned int par_error_word(cudaStream_t st, bool clear);
 
 // ------------------------------------------------------------------ dense projections

@@ -173,6 +173,7 @@ struct ParKArgs {
   float target_alpha[CAST_MAX_FRAMES];
   // bf16 path (tensor cores)
   int n_full;                            // 8x8 tiles (tiles 0 .. n_full-1; the others follow)
+  int after_own;                         // the launch before on the stream is one of this library's kernels
   int n_act, n_grp;                      // pairs with targets; groups of up to two targets of a pair
   int st_parts, st_cpp, bl_parts, bl_cpp;   // K_stats_tc / K_blend_tc: channel-chunk ranges and chunks in each
   // per tile shape (bit 0: last column of tiles, truncated; bit 1: last row): where the stored bin
@@ -739,6 +740,11 @@ __global__ void __launch_bounds__(kStThreads, 1)
     atomicExch(&g_par_error, 1u);
     return false;
   };
+  // Behind a kernel of someone else this CTA takes no TMEM until that one has ended: it may let its
+  // dependents start before its own CTAs have allocated theirs, and would then wait for the columns
+  // of a CTA that waits for its end.  (The attention and the GEMM leave no room for another CTA on
+  // their SM.)
+  if (!a.after_own) grid_dependency_wait();
   if (tid == 0) {
     for (int s = 0; s < kStStages; ++s) {
       mbar_init(&b_full[s], 1);
@@ -1740,7 +1746,7 @@ FastSrc make_fast_src() {
 }
 }  // namespace
 
-cast_status launch_par(const cast_par_args& a, void* ws, cudaStream_t st) {
+cast_status launch_par(const cast_par_args& a, void* ws, cudaStream_t st, bool after_own) {
   const ParPlan p = par_plan(a);
   if (p.n_target == 0) return CAST_OK;   // every frame is an anchor: reconstruction bypassed
   ParKArgs k{};
@@ -1802,6 +1808,7 @@ cast_status launch_par(const cast_par_args& a, void* ws, cudaStream_t st) {
       const int h = (q & 2) ? a.Hg % k.th : k.th, w = (q & 1) ? a.Wg % k.tw : k.tw;
       if (h > 0 && w > 0) make_slots(h, w, k.bin_slot[q], k.slot_bin[q]);
     }
+    k.after_own = after_own ? 1 : 0;
     for (int j = 1; j < na; ++j) {
       if (k.pair_tbeg[j + 1] > k.pair_tbeg[j]) k.act_pair[k.n_act++] = (unsigned char)j;
       for (int t = k.pair_tbeg[j]; t < k.pair_tbeg[j + 1]; t += 2, ++k.n_grp) {
