@@ -172,7 +172,7 @@ struct ParKArgs {
   int target_frame[CAST_MAX_FRAMES];
   float target_alpha[CAST_MAX_FRAMES];
   // bf16 path (tensor cores)
-  int n_full;                            // 8x8 tiles (tiles 0 .. n_full-1; the others follow)
+  int whole_y, whole_x;                  // complete tiles in a column, in a row
   int after_own;                         // the launch before on the stream is one of this library's kernels
   int n_act, n_grp;                      // pairs with targets; groups of up to two targets of a pair
   int st_parts, st_cpp, bl_parts, bl_cpp;   // K_stats_tc / K_blend_tc: channel-chunk ranges and chunks in each
@@ -690,19 +690,32 @@ __device__ void build_dft_operand(const ParKArgs& a, const TileGeom& g, uint8_t*
   }
 }
 
-// One anchor's tile of 128 channels into [64-channel half][8 y + x] of shared memory.  Tiles of
-// other sides than 8x8 are loaded row by row, so that no token of a neighbouring tile is read; the
-// other tokens of their stages are zero (zero_stages, once per CTA) and stay so.
+// One anchor's tile of 128 channels into [64-channel half][8 y + x] of shared memory, one box per
+// half: tiles of eight columns come from the map [frame][row][column], narrower ones from a map
+// [frame][row][tile][column of the tile] with a box of eight columns, whose columns past the tile's
+// side are out of range and arrive as zeros (no token of a neighbouring tile is read).  The last,
+// truncated column of narrower tiles is loaded row by row.  Rows past the tile's side, and here the
+// columns, are not written: they are zero (zero_stages, once per CTA) and stay so.  Row by row for
+// every tile, one thread issued up to 32 copies a chunk: HY-World-shaped PAR took 335 us with 8x4
+// tiles, 242 us with 8x6 and 267 us with 7x5, with boxes 234, 199 and 198 us.
+struct TileMaps {
+  const CUtensorMap *box, *row;   // a tile; one row of it
+};
 __device__ __forceinline__ bool whole_tiles(const ParKArgs& a) { return a.th == 8 && a.tw == 8; }
-__device__ __forceinline__ uint32_t anchor_tile_bytes(const ParKArgs& a) { return (uint32_t)(2 * a.th * a.tw * 128); }
-__device__ __forceinline__ void load_anchor_tile(const ParKArgs& a, const CUtensorMap* tm, uint8_t* dst, uint64_t* bar,
+__device__ __forceinline__ bool boxed(const ParKArgs& a, const TileGeom& g) { return a.tw == 8 || g.w == a.tw; }
+__device__ __forceinline__ uint32_t anchor_tile_bytes(const ParKArgs& a, const TileGeom& g) {
+  return (uint32_t)(2 * a.th * (boxed(a, g) ? 8 : a.tw) * 128);
+}
+__device__ __forceinline__ void load_anchor_tile(const ParKArgs& a, const TileMaps& tm, uint8_t* dst, uint64_t* bar,
                                                  int ch, const TileGeom& g, int frame) {
   for (int b = 0; b < 2; ++b) {
-    if (whole_tiles(a)) {
-      tma_load_4d(dst + b * 8192, tm, bar, ch + b * 64, g.x0, g.y0, frame);
+    if (a.tw == 8) {
+      tma_load_4d(dst + b * 8192, tm.box, bar, ch + b * 64, g.x0, g.y0, frame);
+    } else if (g.w == a.tw) {
+      tma_load_5d(dst + b * 8192, tm.box, bar, ch + b * 64, 0, g.x0 / a.tw, g.y0, frame);
     } else {
       for (int y = 0; y < a.th; ++y)
-        tma_load_4d(dst + b * 8192 + y * 1024, tm, bar, ch + b * 64, g.x0, g.y0 + y, frame);
+        tma_load_4d(dst + b * 8192 + y * 1024, tm.row, bar, ch + b * 64, g.x0, g.y0 + y, frame);
     }
   }
 }
@@ -712,13 +725,35 @@ __device__ __forceinline__ void zero_stages(const ParKArgs& a, uint8_t* p, int b
   fence_proxy_async_smem();
 }
 
-__device__ __forceinline__ TileGeom any_tile(const ParKArgs& a, int tile) {
-  return tile < a.n_full ? tile_geom(a, tile, true) : tile_geom(a, tile - a.n_full, false);
+// Tile i of the bf16 kernels: the complete tiles (row-major), then the truncated last column of every
+// tile row, then the truncated last row, so that tiles of one shape follow one another (a CTA that
+// comes to another shape builds its operand and twiddles anew: row-major over all tiles, the
+// Matrix-Game-shaped PAR took 70 us with 7x5 tiles, 57 us in this order).
+__device__ __forceinline__ TileGeom any_tile(const ParKArgs& a, int i) {
+  const int n = a.whole_y * a.whole_x;
+  int ty, tx;
+  if (i < n) {
+    ty = i / a.whole_x;
+    tx = i - ty * a.whole_x;
+  } else if (a.whole_x < a.tiles_x && i - n < a.tiles_y) {
+    ty = i - n;
+    tx = a.whole_x;
+  } else {
+    ty = a.whole_y;
+    tx = i - n - (a.whole_x < a.tiles_x ? a.tiles_y : 0);
+  }
+  TileGeom g;
+  g.y0 = ty * a.th;
+  g.x0 = tx * a.tw;
+  g.h = min(a.th, a.Hg - g.y0);
+  g.w = min(a.tw, a.Wg - g.x0);
+  return g;
 }
 
 template <bool WEIGHTED>
 __global__ void __launch_bounds__(kStThreads, 1)
-    k_par_stats_tc(const __grid_constant__ CUtensorMap tm, const __grid_constant__ ParKArgs a) {
+    k_par_stats_tc(const __grid_constant__ CUtensorMap tm_box, const __grid_constant__ CUtensorMap tm_row,
+                   const __grid_constant__ ParKArgs a) {
   extern __shared__ uint8_t dsm_raw[];
   const uint32_t raw_addr = smem_u32(dsm_raw);
   uint8_t* dsm = dsm_raw + (((raw_addr + 1023u) & ~1023u) - raw_addr);
@@ -789,7 +824,8 @@ __global__ void __launch_bounds__(kStThreads, 1)
   if (warp < 4) {
     if (warp == 0 && lane == 0) {
       // -------------------------------------------------------------- anchor producer
-      tma_prefetch_desc(&tm);
+      const TileMaps tm{&tm_box, &tm_row};
+      tma_prefetch_desc(&tm_box);
       grid_dependency_wait();   // the anchors (what the sums need besides comes after them)
       int n = 0;
       bool ok = true;
@@ -799,9 +835,9 @@ __global__ void __launch_bounds__(kStThreads, 1)
         for (int c = x.c0; c < x.c1; ++c, ++n) {
           const int s = n % kStStages;
           if (n >= kStStages && !wait(&b_empty[s], (uint32_t)((n / kStStages) - 1) & 1u)) { ok = false; break; }
-          mbar_arrive_expect_tx(&b_full[s], 2 * anchor_tile_bytes(a));
+          mbar_arrive_expect_tx(&b_full[s], 2 * anchor_tile_bytes(a, g));
           for (int q = 0; q < 2; ++q)
-            load_anchor_tile(a, &tm, s_x + (2 * s + q) * kStTile, &b_full[s], c * 128, g, a.anchor_frame[x.j - 1 + q]);
+            load_anchor_tile(a, tm, s_x + (2 * s + q) * kStTile, &b_full[s], c * 128, g, a.anchor_frame[x.j - 1 + q]);
         }
       }
       if (!ok)   // the copies still in flight land before the shared memory is released
@@ -1130,8 +1166,8 @@ constexpr int kTbSmem = kTbStages * kTbStage + 16 * kTbOut + (int)sizeof(MatrixS
 __device__ __forceinline__ void matrix_sync() { asm volatile("bar.sync 3, 128;" ::: "memory"); }
 
 __global__ void __launch_bounds__(kTbThreads, 1)
-    k_par_blend_tc(const __grid_constant__ CUtensorMap tm, const __grid_constant__ CUtensorMap tm_out,
-                   const __grid_constant__ ParKArgs a) {
+    k_par_blend_tc(const __grid_constant__ CUtensorMap tm_box, const __grid_constant__ CUtensorMap tm_row,
+                   const __grid_constant__ CUtensorMap tm_out, const __grid_constant__ ParKArgs a) {
   extern __shared__ uint8_t dsm_raw[];
   const uint32_t raw_addr = smem_u32(dsm_raw);
   uint8_t* dsm = dsm_raw + (((raw_addr + 1023u) & ~1023u) - raw_addr);   // 128-byte swizzle atoms
@@ -1199,7 +1235,8 @@ __global__ void __launch_bounds__(kTbThreads, 1)
   if (warp == 0) {
     if (lane == 0) {
       // -------------------------------------------------------------- anchor producer
-      tma_prefetch_desc(&tm);
+      const TileMaps tm{&tm_box, &tm_row};
+      tma_prefetch_desc(&tm_box);
       // the anchors may come from the launch before the statistics, whose grid waited for it
       grid_dependency_wait();
       int n = 0;
@@ -1211,9 +1248,9 @@ __global__ void __launch_bounds__(kTbThreads, 1)
         for (int c = x.c0; c < x.c1; ++c, ++n) {
           const int s = n % kTbStages;
           if (n >= kTbStages && !wait(&b_xempty[s], (uint32_t)((n / kTbStages) - 1) & 1u)) { ok = false; break; }
-          mbar_arrive_expect_tx(&b_xfull[s], 2 * anchor_tile_bytes(a));
+          mbar_arrive_expect_tx(&b_xfull[s], 2 * anchor_tile_bytes(a, g));
           for (int q = 0; q < 2; ++q)
-            load_anchor_tile(a, &tm, s_x + s * kTbStage + q * kTbPlane, &b_xfull[s], c * 128, g, a.anchor_frame[j - 1 + q]);
+            load_anchor_tile(a, tm, s_x + s * kTbStage + q * kTbPlane, &b_xfull[s], c * 128, g, a.anchor_frame[j - 1 + q]);
         }
       }
       if (!ok)   // the copies still in flight land before the shared memory is released
@@ -1401,7 +1438,7 @@ __global__ void __launch_bounds__(kTbThreads, 1)
     const int set = (warp - 4) >> 2, q = warp & 3;   // TMEM lanes 32 q .. 32 q + 31
     const int ts = q >> 1;                           // target slot of this warp
     const int o = 32 * (q & 1) + lane, yo = o >> 3, xo = o & 7;   // output token 8 y + x
-    const bool valid = yo < a.th && xo < a.tw, whole = a.th == 8 && a.tw == 8;
+    const bool valid = yo < a.th && xo < a.tw, four = a.th >= 4 * (q & 1) + 4;   // four rows of the tile are this warp's
     uint8_t* out0 = s_out + (warp - 4) * 2 * kTbOut;   // two tiles, row yo & 3 at 1 KB each
     const int doff = (yo & 3) * 1024 + xo * 128;
     int n = 0;
@@ -1444,11 +1481,12 @@ __global__ void __launch_bounds__(kTbThreads, 1)
           __syncwarp();
           const int ch = c * 128 + 64 * half;
           if (lane == 0) {
-            if (mine && ch < a.C && whole) {   // four rows of eight tokens
-              if (y0 < a.Hg) tma_store_4d(&tm_out, out, ch, g.x0, y0, frame);
-            } else if (mine && ch < a.C) {     // smaller tiles: one row at a time
+            if (mine && ch < a.C && four && boxed(a, g)) {   // four rows at once
+              if (y0 < a.Hg && a.tw == 8) tma_store_4d(&tm_out, out, ch, g.x0, y0, frame);
+              else if (y0 < a.Hg) tma_store_5d(&tm_out, out, ch, 0, g.x0 / a.tw, y0, frame);
+            } else if (mine && ch < a.C) {   // the last rows of a tile, or a truncated column: one row at a time
               for (int yy = 4 * (q & 1); yy < min(a.th, 4 * (q & 1) + 4) && g.y0 + yy < a.Hg; ++yy)
-                tma_store_4d(&tm_out, out + (yy & 3) * 1024, ch, g.x0, g.y0 + yy, frame);
+                tma_store_4d(&tm_row, out + (yy & 3) * 1024, ch, g.x0, g.y0 + yy, frame);
             }
             bulk_commit();   // one group per half, also where nothing is stored
           }
@@ -1475,6 +1513,21 @@ bool make_r_map_sw(CUtensorMap* m, const cast_par_args& a, int bw, int bh) {
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// 5-D map [F][Hg][complete tiles of a row][column of a tile][C] with a 128-byte-swizzled box (64 bf16
+// channels, 8 columns, 1, bh, 1)
+bool make_tile_map_sw(CUtensorMap* m, const cast_par_args& a, int bh) {
+  EncodeTiledFn fn = tensor_map_encoder();
+  if (!fn) return false;
+  const cuuint64_t tw = (cuuint64_t)a.params.tile_w, token = a.C * 2ull;
+  cuuint64_t dims[5] = {(cuuint64_t)a.C, tw, (cuuint64_t)a.Wg / tw, (cuuint64_t)a.Hg, (cuuint64_t)a.F};
+  cuuint64_t strides[4] = {token, tw * token, a.Wg * token, (cuuint64_t)a.Hg * a.Wg * token};
+  cuuint32_t box[5] = {64, 8, 1, (cuuint32_t)bh, 1};
+  cuuint32_t es[5] = {1, 1, 1, 1, 1};
+  return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, a.r, dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
+            CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 // 4-D map [F][Hg][Wg][C], box (cc channels, tw, th, 1), zero fill out of range
 bool make_r_map(CUtensorMap* m, const cast_par_args& a, int cc) {
   EncodeTiledFn fn = tensor_map_encoder();
@@ -1491,7 +1544,8 @@ bool make_r_map(CUtensorMap* m, const cast_par_args& a, int cc) {
 
 // bf16: two launches over every tile, each a programmatic dependent of the launch before it on the
 // stream (the statistics kernel sets itself up and builds its operand while that one ends).
-cast_status launch_tc(const CUtensorMap& tm_sw, const CUtensorMap& tm_out, const ParKArgs& k, cudaStream_t st) {
+cast_status launch_tc(const CUtensorMap& tm_box, const CUtensorMap& tm_row, const CUtensorMap& tm_out, const ParKArgs& k,
+                      cudaStream_t st) {
   static std::atomic<uint64_t> attr_done{0};
   if (!once_per_device(attr_done, [] {
         return cudaFuncSetAttribute(k_par_stats_tc<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kStSmem) ==
@@ -1512,7 +1566,8 @@ cast_status launch_tc(const CUtensorMap& tm_sw, const CUtensorMap& tm_out, const
   cfg.stream = st;
   cfg.attrs = pdl;
   cfg.numAttrs = 1;
-  if (cudaLaunchKernelEx(&cfg, k.wch ? k_par_stats_tc<true> : k_par_stats_tc<false>, tm_sw, k) != cudaSuccess) return check_launch("PAR statistics kernel");
+  if (cudaLaunchKernelEx(&cfg, k.wch ? k_par_stats_tc<true> : k_par_stats_tc<false>, tm_box, tm_row, k) != cudaSuccess)
+    return check_launch("PAR statistics kernel");
   cudaLaunchConfig_t bc{};
   bc.gridDim = dim3(std::min(k.n_tile * k.n_grp * k.bl_parts, sm_count()), 1, 1);
   bc.blockDim = dim3(kTbThreads, 1, 1);
@@ -1520,7 +1575,7 @@ cast_status launch_tc(const CUtensorMap& tm_sw, const CUtensorMap& tm_out, const
   bc.stream = st;
   bc.attrs = pdl;
   bc.numAttrs = 1;
-  if (cudaLaunchKernelEx(&bc, k_par_blend_tc, tm_sw, tm_out, k) != cudaSuccess)
+  if (cudaLaunchKernelEx(&bc, k_par_blend_tc, tm_box, tm_row, tm_out, k) != cudaSuccess)
     return check_launch("PAR tensor-core blend kernel");
   return check_launch("PAR kernels");
 }
@@ -1803,7 +1858,8 @@ cast_status launch_par(const cast_par_args& a, void* ws, cudaStream_t st, bool a
   std::copy(fast_src.v, fast_src.v + kNV, k.fast_src);
 
   if (a.dtype == CAST_BF16) {
-    k.n_full = p.n_full;
+    k.whole_y = a.Hg / k.th;
+    k.whole_x = a.Wg / k.tw;
     for (int q = 0; q < 4; ++q) {
       const int h = (q & 2) ? a.Hg % k.th : k.th, w = (q & 1) ? a.Wg % k.tw : k.tw;
       if (h > 0 && w > 0) make_slots(h, w, k.bin_slot[q], k.slot_bin[q]);
@@ -1840,12 +1896,17 @@ cast_status launch_par(const cast_par_args& a, void* ws, cudaStream_t st, bool a
     };
     split((int64_t)p.n_tile * k.n_act, 1, 0, 4, k.st_parts, k.st_cpp);
     split((int64_t)p.n_tile * k.n_grp, 0, 6, 8, k.bl_parts, k.bl_cpp);
-    CUtensorMap tm_sw, tm_out;
-    // anchors in boxes of 8 x 8 tokens, outputs in four rows of a tile; other tile sides row by row
-    const bool whole = k.th == 8 && k.tw == 8;
-    if (!make_r_map_sw(&tm_sw, a, k.tw, whole ? 8 : 1) || !make_r_map_sw(&tm_out, a, k.tw, whole ? 4 : 1))
-      return fail(CAST_ERR_CUDA, "PAR: cuTensorMapEncodeTiled failed");
-    return launch_tc(tm_sw, tm_out, k, st);
+    CUtensorMap tm_box, tm_row, tm_out;
+    bool ok = make_r_map_sw(&tm_row, a, k.tw, 1);
+    if (k.tw == 8) {
+      ok = ok && make_r_map_sw(&tm_box, a, 8, k.th) && make_r_map_sw(&tm_out, a, 8, 4);
+    } else if (a.Wg >= k.tw) {
+      ok = ok && make_tile_map_sw(&tm_box, a, k.th) && make_tile_map_sw(&tm_out, a, 4);
+    } else {   // no complete tile in a row: everything row by row
+      tm_box = tm_out = tm_row;
+    }
+    if (!ok) return fail(CAST_ERR_CUDA, "PAR: cuTensorMapEncodeTiled failed");
+    return launch_tc(tm_box, tm_row, tm_out, k, st);
   }
   CUtensorMap tm;
   if (!make_r_map(&tm, a, p.chunk)) return fail(CAST_ERR_CUDA, "PAR: cuTensorMapEncodeTiled failed");
