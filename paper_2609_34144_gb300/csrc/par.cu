@@ -158,6 +158,12 @@ __host__ __device__ __forceinline__ constexpr int fast_value(int n) {
       0;
 }
 
+// A unit of the bf16 kernels: a tile, a range of its channel chunks and an item (a pair, or a group of
+// targets), items innermost, so that a tile's anchors are read from L2 by the CTAs of neighbouring units.
+struct Unit {
+  int tile, part, item;
+};
+
 struct ParKArgs {
   char* r;
   const float* wch;
@@ -176,6 +182,7 @@ struct ParKArgs {
   int after_own;                         // the launch before on the stream is one of this library's kernels
   int n_act, n_grp;                      // pairs with targets; groups of up to two targets of a pair
   int st_parts, st_cpp, bl_parts, bl_cpp;   // K_stats_tc / K_blend_tc: channel-chunk ranges and chunks in each
+  Unit st_step, bl_step;                 // ... and the CTAs' stride over the units
   // per tile shape (bit 0: last column of tiles, truncated; bit 1: last row): where the stored bin
   // b's sums stand in a record (BinSlot), and the bin of each slot (255: none)
   unsigned char bin_slot[4][40], slot_bin[4][34];
@@ -301,10 +308,10 @@ __device__ void bin_info(const ParKArgs& a, const TileGeom& g, BinInfo& bi, int 
   bi.cut[b] = cut;
 }
 
-// Per-tile transport of one anchor pair (warp 0, two bins per lane): theta and g per stored
-// bin from the pooled Z, W record (App. A.2).
+// Per-tile transport of one anchor pair (one warp): theta and g of the stored bins lane and
+// lane + 32 from the pooled Z, W record (App. A.2).
 __device__ void tile_transport(const ParKArgs& a, const TileGeom& g, const BinInfo& bi,
-                               const float* zw, float* th, float* gate, float* own_th,
+                               const float* zw, float (&th)[2], float (&gate)[2], float* own_th,
                                int* own_rel, int lane) {
   const float inv_hw = 1.f / (float)(g.h * g.w);
   float Zr[2], Zi[2], Wv[2], Za[2], t[2];
@@ -363,14 +370,15 @@ __device__ void tile_transport(const ParKArgs& a, const TileGeom& g, const BinIn
 #pragma unroll
   for (int s = 0; s < 2; ++s) {
     const int b = lane + 32 * s;
+    th[s] = gate[s] = 0.f;
     if (b >= kNB) continue;
     const float tau = bi.tau[b];
     float gv = rcp_approx(1.f + __expf((tau - c) * rcp_approx(a.T)));
     if (a.gate_mode == CAST_GATE_ZERO) gv = 0.f;
     if (a.gate_mode == CAST_GATE_ONE) gv = 1.f;
     if (bi.cut[b]) gv = 0.f;   // outside the band
-    th[b] = any ? thv[s] : 0.f;
-    gate[b] = gv;
+    th[s] = any ? thv[s] : 0.f;
+    gate[s] = gv;
   }
 }
 
@@ -750,6 +758,26 @@ __device__ __forceinline__ TileGeom any_tile(const ParKArgs& a, int i) {
   return g;
 }
 
+// The units of a CTA: blockIdx.x, then every gridDim.x-th.  Stepping in (tile, part, item) costs no
+// division: the divisions took ~1,000 cycles of every role and unit, and a unit of one channel chunk has
+// ~1,100 cycles of work in the statistics (16 frames of 44x80 x 64 channels: 6x6 tiles 42 -> 40 us, 4x4
+// tiles 59 -> 54 us).
+__device__ __forceinline__ Unit first_unit(int n_part, int n_item) {
+  Unit u;
+  const int q = blockIdx.x / n_item;
+  u.item = blockIdx.x - q * n_item;
+  u.tile = q / n_part;
+  u.part = q - u.tile * n_part;
+  return u;
+}
+__device__ __forceinline__ void next_unit(Unit& u, const Unit& step, int n_part, int n_item) {
+  u.item += step.item;
+  u.part += step.part;
+  u.tile += step.tile;
+  if (u.item >= n_item) u.item -= n_item, ++u.part;
+  if (u.part >= n_part) u.part -= n_part, ++u.tile;
+}
+
 template <bool WEIGHTED>
 __global__ void __launch_bounds__(kStThreads, 1)
     k_par_stats_tc(const __grid_constant__ CUtensorMap tm_box, const __grid_constant__ CUtensorMap tm_row,
@@ -765,7 +793,6 @@ __global__ void __launch_bounds__(kStThreads, 1)
   __shared__ uint32_t s_tmem;
   __shared__ volatile int s_abort;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int nck = a.n_chunk, n_units = a.n_tile * a.n_act * a.st_parts;
   const uint64_t lim = a.wait_ns;
   auto wait = [&](uint64_t* bar, uint32_t parity) -> bool {
     if (mbar_try_wait(bar, parity)) return true;
@@ -804,22 +831,9 @@ __global__ void __launch_bounds__(kStThreads, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = s_tmem;
-  // unit u -> (tile, pair, chunk range): pairs innermost, so that a tile's anchors are read
-  // from L2 by the CTAs of neighbouring units
-  struct Unit {
-    int tile, j, part, c0, c1;
-  };
-  auto unit_of = [&](int u) {
-    Unit x;
-    const int per = a.n_act * a.st_parts;
-    x.tile = u / per;
-    const int r = u - x.tile * per;
-    x.part = r / a.n_act;
-    x.j = a.act_pair[r - x.part * a.n_act];
-    x.c0 = x.part * a.st_cpp;
-    x.c1 = min(nck, x.c0 + a.st_cpp);
-    return x;
-  };
+  const int nck = a.n_chunk, n_part = a.st_parts, n_item = a.n_act;   // an item: a pair with targets
+  const auto c0_of = [&](const Unit& u) { return u.part * a.st_cpp; };
+  const auto c1_of = [&](const Unit& u) { return min(nck, (u.part + 1) * a.st_cpp); };
 
   if (warp < 4) {
     if (warp == 0 && lane == 0) {
@@ -829,15 +843,14 @@ __global__ void __launch_bounds__(kStThreads, 1)
       grid_dependency_wait();   // the anchors (what the sums need besides comes after them)
       int n = 0;
       bool ok = true;
-      for (int u = blockIdx.x; ok && u < n_units; u += gridDim.x) {
-        const Unit x = unit_of(u);
+      for (Unit x = first_unit(n_part, n_item); ok && x.tile < a.n_tile; next_unit(x, a.st_step, n_part, n_item)) {
         const TileGeom g = any_tile(a, x.tile);
-        for (int c = x.c0; c < x.c1; ++c, ++n) {
+        for (int c = c0_of(x), c1 = c1_of(x); c < c1; ++c, ++n) {
           const int s = n % kStStages;
           if (n >= kStStages && !wait(&b_empty[s], (uint32_t)((n / kStStages) - 1) & 1u)) { ok = false; break; }
           mbar_arrive_expect_tx(&b_full[s], 2 * anchor_tile_bytes(a, g));
           for (int q = 0; q < 2; ++q)
-            load_anchor_tile(a, tm, s_x + (2 * s + q) * kStTile, &b_full[s], c * 128, g, a.anchor_frame[x.j - 1 + q]);
+            load_anchor_tile(a, tm, s_x + (2 * s + q) * kStTile, &b_full[s], c * 128, g, a.anchor_frame[a.act_pair[x.item] - 1 + q]);
         }
       }
       if (!ok)   // the copies still in flight land before the shared memory is released
@@ -855,8 +868,7 @@ __global__ void __launch_bounds__(kStThreads, 1)
       const bool lead = elect_one();
       int n = 0, last = -1, shape = -1, builds = 0;
       bool ok = true;
-      for (int u = blockIdx.x; ok && u < n_units; u += gridDim.x) {
-        const Unit x = unit_of(u);
+      for (Unit x = first_unit(n_part, n_item); ok && x.tile < a.n_tile; next_unit(x, a.st_step, n_part, n_item)) {
         const TileGeom g = any_tile(a, x.tile);
         if (g.h * 16 + g.w != shape) {
           shape = g.h * 16 + g.w;
@@ -864,7 +876,7 @@ __global__ void __launch_bounds__(kStThreads, 1)
           if (lane == 0) mbar_arrive(&b_seen);
         }
         const bool pieces = !(g.h == 8 && g.w == 8);
-        for (int c = x.c0; c < x.c1; ++c, ++n) {
+        for (int c = c0_of(x), c1 = c1_of(x); c < c1; ++c, ++n) {
           if ((n & 1) != buf) continue;
           const int s = n % kStStages;
           // half of the warp waits for the anchors, half for the accumulator
@@ -907,8 +919,7 @@ __global__ void __launch_bounds__(kStThreads, 1)
     constexpr float kR = 0.70710678118654752f;
     int n = 0, shape = 0, flip = 0;   // shape: operands built so far << 8 | sides of the last one
     bool ok = true;
-    for (int u = blockIdx.x; u < n_units; u += gridDim.x, flip ^= 1) {
-      const Unit x = unit_of(u);
+    for (Unit x = first_unit(n_part, n_item); x.tile < a.n_tile; next_unit(x, a.st_step, n_part, n_item), flip ^= 1) {
       const TileGeom g = any_tile(a, x.tile);
       if (g.h * 16 + g.w != (shape & 255)) {
         // every UMMA that read the operand has completed: its chunk has been waited for
@@ -941,7 +952,7 @@ __global__ void __launch_bounds__(kStThreads, 1)
           wv[s] += aw;
         }
       };
-      for (int c = x.c0; c < x.c1; ++c, ++n) {
+      for (int c = c0_of(x), c1 = c1_of(x); c < c1; ++c, ++n) {
         const int buf = n & 1, ch = c * 128 + q4 * 32 + lane;
         if (!(ok = __all_sync(0xffffffffu, wait(&b_dfull[buf], (uint32_t)(n >> 1) & 1u)))) break;
         tc_fence_after();
@@ -1004,7 +1015,7 @@ __global__ void __launch_bounds__(kStThreads, 1)
         float sum = 0.f;
 #pragma unroll
         for (int w4 = 0; w4 < 4; ++w4) sum += s_red[(flip * kStSumWarps + of * 4 + w4) * 32 + at];
-        a.rec[(((int64_t)x.tile * a.n_anchor + x.j) * a.n_chunk + x.part) * kRec + ctid] = sum;
+        a.rec[(((int64_t)x.tile * a.n_anchor + a.act_pair[x.item]) * a.n_chunk + x.part) * kRec + ctid] = sum;
       }
       // the other half of s_red is written next, this one only after the next unit's barrier
     }
@@ -1032,7 +1043,7 @@ __device__ __forceinline__ float record_sum(const float* r, int n) {
 template <bool FULL>
 __global__ void __launch_bounds__(128) k_par_transport(const __grid_constant__ ParKArgs a) {
   __shared__ float s_zw[kNV];
-  __shared__ float s_th[kNB], s_g[kNB], s_own_th[kNB];
+  __shared__ float s_own_th[kNB];
   __shared__ int s_own_rel[kNB];
   __shared__ BinInfo s_bins;
   const int tid = threadIdx.x;
@@ -1056,12 +1067,18 @@ __global__ void __launch_bounds__(128) k_par_transport(const __grid_constant__ P
     s_zw[tid] = sign < 0 ? -sum : sum;
   }
   __syncthreads();
-  if (tid < 32) tile_transport(a, g, s_bins, s_zw, s_th, s_g, s_own_th, s_own_rel, tid);
-  __syncthreads();
-  if (tid < kNB) {
+  if (tid < 32) {
+    float th[2], gate[2];
+    tile_transport(a, g, s_bins, s_zw, th, gate, s_own_th, s_own_rel, tid);
     float* tr = a.trans + ((int64_t)tg * a.n_anchor + j) * 2 * kNB;
-    tr[tid] = s_th[tid];
-    tr[kNB + tid] = s_g[tid];
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+      const int b = tid + 32 * s;
+      if (b < kNB) {
+        tr[b] = th[s];
+        tr[kNB + b] = gate[s];
+      }
+    }
   }
   launch_dependents();
 }
@@ -1102,44 +1119,44 @@ struct TransportShared {
   int own_rel[kNB];
   unsigned char slot[kNB];
 };
-__device__ void transport_shape(const ParKArgs& a, const TileGeom& g, TransportShared& m, int lane) {
+constexpr int kZwPer = (kNV + 31) / 32;   // entries of zw per lane: lane, lane + 32, ...
+__device__ void transport_shape(const ParKArgs& a, const TileGeom& g, TransportShared& m, int (&at)[kZwPer], int lane) {
 #pragma unroll 1
   for (int b = lane; b < kNB; b += 32) {
     bin_info(a, g, m.bins, b);
     m.slot[b] = a.bin_slot[tile_shape(a, g)][b];
   }
   __syncwarp();
-}
-__device__ void unit_transport(const ParKArgs& a, const TileGeom& g, int tile, int j, TransportShared& m, float* th,
-                               float* gate, int lane) {
-  const float* rec = a.rec + ((int64_t)tile * a.n_anchor + j) * a.n_chunk * kRec;
-  // four entries per lane, summed over the parts in order, sixteen loads in flight
-  constexpr int kPer = (kNV + 31) / 32;
-  int at[kPer];
-  float sum[kPer];
 #pragma unroll
-  for (int i = 0; i < kPer; ++i) {
+  for (int i = 0; i < kZwPer; ++i) {
     const int e = lane + 32 * i, b = min(e / 3, kNB - 1), comp = e - 3 * (e / 3), code = m.slot[b], slot = code & 63;
     // Re Z, Im Z, W of complex slot s stand at s, 30 + s, 60 + s, Z and W of real slot s at 90 + s, 94 + s
     at[i] = comp * kNCpx + slot;
     if (code & kSlotReal) at[i] = comp == 1 ? -1 : 3 * kNCpx + (comp == 2 ? kNReal : 0) + slot;
     if (code == 255 || e >= kNV) at[i] = -1;
-    sum[i] = 0.f;
   }
-  for (int q0 = 0; q0 < a.st_parts; q0 += 4) {
-    float v[kPer][4];
+}
+__device__ void unit_transport(const ParKArgs& a, const TileGeom& g, int tile, int j, TransportShared& m,
+                               const int (&at)[kZwPer], float (&th)[2], float (&gate)[2], int lane) {
+  const float* rec = a.rec + ((int64_t)tile * a.n_anchor + j) * a.n_chunk * kRec;
+  // this lane's entries, summed over the parts in order, sixteen loads in flight
+  float sum[kZwPer];
 #pragma unroll
-    for (int i = 0; i < kPer; ++i)
+  for (int i = 0; i < kZwPer; ++i) sum[i] = 0.f;
+  for (int q0 = 0; q0 < a.st_parts; q0 += 4) {
+    float v[kZwPer][4];
+#pragma unroll
+    for (int i = 0; i < kZwPer; ++i)
 #pragma unroll
       for (int q = 0; q < 4; ++q)
         v[i][q] = at[i] >= 0 && q0 + q < a.st_parts ? __ldcg(rec + (int64_t)(q0 + q) * kRec + at[i]) : 0.f;
 #pragma unroll
-    for (int i = 0; i < kPer; ++i)
+    for (int i = 0; i < kZwPer; ++i)
 #pragma unroll
       for (int q = 0; q < 4; ++q) sum[i] += v[i][q];
   }
 #pragma unroll
-  for (int i = 0; i < kPer; ++i) {
+  for (int i = 0; i < kZwPer; ++i) {
     const int e = lane + 32 * i;
     if (e < kNV) m.zw[e] = (e % 3) == 1 && (m.slot[e / 3] & kSlotMirror) && at[i] >= 0 ? -sum[i] : sum[i];
   }
@@ -1180,7 +1197,6 @@ __global__ void __launch_bounds__(kTbThreads, 1)
   __shared__ uint32_t s_tmem;
   __shared__ volatile int s_abort;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int n_units = a.n_tile * a.n_grp * a.bl_parts;
   const uint64_t lim = a.wait_ns;
   auto wait = [&](uint64_t* bar, uint32_t parity) -> bool {
     if (mbar_try_wait(bar, parity)) return true;
@@ -1216,21 +1232,9 @@ __global__ void __launch_bounds__(kTbThreads, 1)
   tc_fence_after();
   const uint32_t tmem = s_tmem;
   // (the warps that read what earlier launches wrote, 0 and 2, wait for the grid before)
-  // unit u -> (tile, target group, chunk range): groups innermost, so that a tile's anchors are
-  // read from L2 by the CTAs of neighbouring units
-  struct Unit {
-    int tile, grp, c0, c1;
-  };
-  auto unit_of = [&](int u) {
-    Unit x;
-    const int per = a.n_grp * a.bl_parts;
-    x.tile = u / per;
-    const int r = u - x.tile * per, part = r / a.n_grp;
-    x.grp = r - part * a.n_grp;
-    x.c0 = part * a.bl_cpp;
-    x.c1 = min(a.n_chunk, x.c0 + a.bl_cpp);
-    return x;
-  };
+  const int n_part = a.bl_parts, n_item = a.n_grp;   // an item: up to two targets of a pair
+  const auto c0_of = [&](const Unit& u) { return u.part * a.bl_cpp; };
+  const auto c1_of = [&](const Unit& u) { return min(a.n_chunk, (u.part + 1) * a.bl_cpp); };
 
   if (warp == 0) {
     if (lane == 0) {
@@ -1241,11 +1245,10 @@ __global__ void __launch_bounds__(kTbThreads, 1)
       grid_dependency_wait();
       int n = 0;
       bool ok = true;
-      for (int u = blockIdx.x; ok && u < n_units; u += gridDim.x) {
-        const Unit x = unit_of(u);
+      for (Unit x = first_unit(n_part, n_item); ok && x.tile < a.n_tile; next_unit(x, a.bl_step, n_part, n_item)) {
         const TileGeom g = any_tile(a, x.tile);
-        const int j = a.grp_pair[x.grp];
-        for (int c = x.c0; c < x.c1; ++c, ++n) {
+        const int j = a.grp_pair[x.item];
+        for (int c = c0_of(x), c1 = c1_of(x); c < c1; ++c, ++n) {
           const int s = n % kTbStages;
           if (n >= kTbStages && !wait(&b_xempty[s], (uint32_t)((n / kTbStages) - 1) & 1u)) { ok = false; break; }
           mbar_arrive_expect_tx(&b_xfull[s], 2 * anchor_tile_bytes(a, g));
@@ -1265,10 +1268,9 @@ __global__ void __launch_bounds__(kTbThreads, 1)
     const uint32_t tm = tmem + ((uint32_t)((warp & 3) * 32) << 16);
     int k = 0, shape = -1;
     float2 twx[5], twy[8];   // e^{2 pi i kx dx / w}, e^{2 pi i ky dy / h}; 0 past the stored bins
-    for (int u = blockIdx.x; u < n_units; u += gridDim.x, ++k) {
-      const Unit x = unit_of(u);
+    for (Unit x = first_unit(n_part, n_item); x.tile < a.n_tile; next_unit(x, a.bl_step, n_part, n_item), ++k) {
       const TileGeom g = any_tile(a, x.tile);
-      const int h = g.h, w = g.w, t0 = a.grp_t0[x.grp], nt = a.grp_nt[x.grp];
+      const int h = g.h, w = g.w, t0 = a.grp_t0[x.item], nt = a.grp_nt[x.item];
       if (h * 16 + w != shape) {
         shape = h * 16 + w;
 #pragma unroll
@@ -1375,16 +1377,25 @@ __global__ void __launch_bounds__(kTbThreads, 1)
   } else if (warp == 2) {
     // ---------------------------------------------------------------- transport
     __shared__ TransportShared ms;
-    int k = 0, shape = -1;
-    for (int u = blockIdx.x; u < n_units; u += gridDim.x, ++k) {
-      const Unit x = unit_of(u);
+    int k = 0, shape = -1, at[kZwPer];
+    for (Unit x = first_unit(n_part, n_item); x.tile < a.n_tile; next_unit(x, a.bl_step, n_part, n_item), ++k) {
       const TileGeom g = any_tile(a, x.tile);
       const bool fresh = g.h * 16 + g.w != shape;
       shape = g.h * 16 + g.w;
-      if (fresh) transport_shape(a, g, ms, lane);
+      if (fresh) transport_shape(a, g, ms, at, lane);
       if (k == 0) grid_dependency_wait();   // the records of K_stats_tc
+      // only the hand-over waits for the matrix warps to have read the unit before (the transport
+      // takes ~5,000 cycles, their reading of it ~2,000)
+      float th[2], gate[2];
+      unit_transport(a, g, x.tile, a.grp_pair[x.item], ms, at, th, gate, lane);
       if (!__all_sync(0xffffffffu, k == 0 || wait(&b_tfree, (uint32_t)(k - 1) & 1u))) break;
-      unit_transport(a, g, x.tile, a.grp_pair[x.grp], ms, s_th, s_gate, lane);
+#pragma unroll
+      for (int s = 0; s < 2; ++s)
+        if (lane + 32 * s < kNB) {
+          s_th[lane + 32 * s] = th[s];
+          s_gate[lane + 32 * s] = gate[s];
+        }
+      __syncwarp();
       if (lane == 0) mbar_arrive(&b_tready);
     }
   } else if (warp < 4) {
@@ -1398,12 +1409,11 @@ __global__ void __launch_bounds__(kTbThreads, 1)
     const bool lead = elect_one();
     int n = 0, k = 0, last = -1;
     bool ok = true;
-    for (int u = blockIdx.x; ok && u < n_units; u += gridDim.x, ++k) {
-      const Unit x = unit_of(u);
+    for (Unit x = first_unit(n_part, n_item); ok && x.tile < a.n_tile; next_unit(x, a.bl_step, n_part, n_item), ++k) {
       const int mb = k & 1;
       if (!(ok = __all_sync(0xffffffffu, wait(&b_mfull[mb], (uint32_t)(k >> 1) & 1u)))) break;
       tc_fence_after();
-      for (int c = x.c0; c < x.c1; ++c, ++n) {
+      for (int c = c0_of(x), c1 = c1_of(x); c < c1; ++c, ++n) {
         if ((n & 1) != buf) continue;
         const int s = n % kTbStages;
         // half of the warp waits for the anchors, half for the accumulator
@@ -1443,12 +1453,11 @@ __global__ void __launch_bounds__(kTbThreads, 1)
     const int doff = (yo & 3) * 1024 + xo * 128;
     int n = 0;
     bool ok = true;
-    for (int u = blockIdx.x; ok && u < n_units; u += gridDim.x) {
-      const Unit x = unit_of(u);
+    for (Unit x = first_unit(n_part, n_item); ok && x.tile < a.n_tile; next_unit(x, a.bl_step, n_part, n_item)) {
       const TileGeom g = any_tile(a, x.tile);
-      const bool mine = ts < a.grp_nt[x.grp];
-      const int frame = mine ? a.target_frame[a.grp_t0[x.grp] + ts] : 0, y0 = g.y0 + 4 * (q & 1);
-      for (int c = x.c0; c < x.c1; ++c, ++n) {
+      const bool mine = ts < a.grp_nt[x.item];
+      const int frame = mine ? a.target_frame[a.grp_t0[x.item] + ts] : 0, y0 = g.y0 + 4 * (q & 1);
+      for (int c = c0_of(x), c1 = c1_of(x); c < c1; ++c, ++n) {
         if ((n & 1) != set) continue;
         if (!__all_sync(0xffffffffu, wait(&b_dfull[set], (uint32_t)(n >> 1) & 1u))) { ok = false; break; }
         tc_fence_after();
@@ -1544,7 +1553,7 @@ bool make_r_map(CUtensorMap* m, const cast_par_args& a, int cc) {
 
 // bf16: two launches over every tile, each a programmatic dependent of the launch before it on the
 // stream (the statistics kernel sets itself up and builds its operand while that one ends).
-cast_status launch_tc(const CUtensorMap& tm_box, const CUtensorMap& tm_row, const CUtensorMap& tm_out, const ParKArgs& k,
+cast_status launch_tc(const CUtensorMap& tm_box, const CUtensorMap& tm_row, const CUtensorMap& tm_out, ParKArgs& k,
                       cudaStream_t st) {
   static std::atomic<uint64_t> attr_done{0};
   if (!once_per_device(attr_done, [] {
@@ -1559,8 +1568,15 @@ cast_status launch_tc(const CUtensorMap& tm_box, const CUtensorMap& tm_row, cons
   cudaLaunchAttribute pdl[1];
   pdl[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   pdl[0].val.programmaticStreamSerializationAllowed = 1;
+  const auto grid_of = [&](int n_part, int n_item, Unit& step) {   // CTAs, and their stride over the units
+    const int n = (int)std::min<int64_t>((int64_t)k.n_tile * n_part * n_item, sm_count());
+    step.item = n % n_item;
+    step.part = n / n_item % n_part;
+    step.tile = n / n_item / n_part;
+    return dim3(n, 1, 1);
+  };
   cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(std::min(k.n_tile * k.n_act * k.st_parts, sm_count()), 1, 1);
+  cfg.gridDim = grid_of(k.st_parts, k.n_act, k.st_step);
   cfg.blockDim = dim3(kStThreads, 1, 1);
   cfg.dynamicSmemBytes = kStSmem;
   cfg.stream = st;
@@ -1569,7 +1585,7 @@ cast_status launch_tc(const CUtensorMap& tm_box, const CUtensorMap& tm_row, cons
   if (cudaLaunchKernelEx(&cfg, k.wch ? k_par_stats_tc<true> : k_par_stats_tc<false>, tm_box, tm_row, k) != cudaSuccess)
     return check_launch("PAR statistics kernel");
   cudaLaunchConfig_t bc{};
-  bc.gridDim = dim3(std::min(k.n_tile * k.n_grp * k.bl_parts, sm_count()), 1, 1);
+  bc.gridDim = grid_of(k.bl_parts, k.n_grp, k.bl_step);
   bc.blockDim = dim3(kTbThreads, 1, 1);
   bc.dynamicSmemBytes = kTbSmem;
   bc.stream = st;
