@@ -30,8 +30,7 @@
 // cluster barrier at the end keeps both CTAs' shared memory until nothing is in flight.
 #include <cuda_bf16.h>
 
-#include <algorithm>
-
+#include "dense_plan.h"
 #include "internal.h"
 #include "ptx.cuh"
 
@@ -366,18 +365,6 @@ bool make_gemm_map(CUtensorMap* m, const void* base, uint64_t inner, uint64_t ro
   return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, depth ? 3 : 2, const_cast<void*>(base), dims, strides,
             box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
-// Columns per tile: 256, or 128 where 256 would leave SMs without work.  A 64-wide k-step of a
-// pair takes about 660 cycles at 256 columns (32 KB per SM) and 480 at 128 (24 KB; both bound by
-// the ~50 bytes per clock that an SM takes from L2, measured at the Matrix-Game-shaped FFN: 69 and
-// 96 us for its second GEMM), the epilogue of a tile about 16 cycles a column.
-int tile_columns(int row_pairs, int N, int n_k, int pairs) {
-  auto cycles = [&](int bn, int step) -> int64_t {
-    const int64_t items = (int64_t)row_pairs * ((N + bn - 1) / bn), rounds = (items + pairs - 1) / pairs;
-    return rounds * std::max<int64_t>((int64_t)n_k * step, 16 * bn) + 16 * bn;
-  };
-  return cycles(128, 480) < cycles(256, 660) ? 128 : 256;
 }
 
 }  // namespace
