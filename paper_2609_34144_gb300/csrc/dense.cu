@@ -166,7 +166,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGThreads, 1)
           tma_load_2d_pair(st + kABytes, &tm_w, bar, ks * GBK, g.n0 + rank * half_n);
         }
       }
-      if (!ok && rank == 0)   // the copies still in flight land before shared memory is released
+      if (rank == 0)   // (whatever ended the loop) the last copies have landed before shared memory is released
         for (int l = it > kGStages ? it - kGStages : 0; l < it; ++l)
           mbar_wait(&bars->full[l % kGStages], (uint32_t)(l / kGStages) & 1u, lim);
     }

@@ -853,9 +853,9 @@ __global__ void __launch_bounds__(kStThreads, 1)
             load_anchor_tile(a, tm, s_x + (2 * s + q) * kStTile, &b_full[s], c * 128, g, a.anchor_frame[a.act_pair[x.item] - 1 + q]);
         }
       }
-      if (!ok)   // the copies still in flight land before the shared memory is released
-        for (int l = n > kStStages ? n - kStStages : 0; l < n; ++l)
-          mbar_wait(&b_full[l % kStStages], (uint32_t)(l / kStStages) & 1u, lim);
+      // (whatever ended the loop) the last copies have landed before shared memory is released
+      for (int l = n > kStStages ? n - kStStages : 0; l < n; ++l)
+        mbar_wait(&b_full[l % kStStages], (uint32_t)(l / kStStages) & 1u, lim);
     } else if (warp & 1) {
       // -------------------------------------------------------------- UMMA issuers (converged)
       // warps 1 and 3 take alternate chunks and accumulators: the ~500 cycles that an issuer
@@ -1256,9 +1256,8 @@ __global__ void __launch_bounds__(kTbThreads, 1)
             load_anchor_tile(a, tm, s_x + s * kTbStage + q * kTbPlane, &b_xfull[s], c * 128, g, a.anchor_frame[j - 1 + q]);
         }
       }
-      if (!ok)   // the copies still in flight land before the shared memory is released
-        for (int l = n > kTbStages ? n - kTbStages : 0; l < n; ++l)
-          mbar_wait(&b_xfull[l % kTbStages], (uint32_t)(l / kTbStages) & 1u, lim);
+      for (int l = n > kTbStages ? n - kTbStages : 0; l < n; ++l)
+        mbar_wait(&b_xfull[l % kTbStages], (uint32_t)(l / kTbStages) & 1u, lim);
     }
   } else if (warp >= 12) {
     // ---------------------------------------------------------------- matrices
