@@ -118,7 +118,7 @@ struct ParPlan {
   int chunk;        // channels per CTA (= threads per CTA)
   int n_chunk;      // channel chunks per tile
   int n_tseg_full, n_tseg_edge;   // time segments (runs of anchor pairs) per tile, per kind
-  size_t rec_bytes, trans_bytes, total_bytes;   // workspace: chunk records, theta and g
+  size_t rec_bytes, trans_bytes, total_bytes;   // workspace: chunk records; theta and g (f32)
 };
 ParPlan par_plan(const cast_par_args& a);
 // after_own: the launch before on the stream is a kernel of this library (attention or GEMM)

@@ -168,7 +168,7 @@ struct ParKArgs {
   char* r;
   const float* wch;
   float* rec;     // workspace [tile][pair j][chunk][kRec]: each chunk's Z / W record
-  float* trans;   // workspace [tile][pair j][2][kNB]: theta and g per bin
+  float* trans;   // workspace [tile][pair j][2][kNB]: theta and g per bin (f32)
   int F, Hg, Wg, C, n_chunk;             // n_chunk: channel chunks of kCC channels
   int tile_base;                         // global index of tile 0 of this launch's kind
   int th, tw, tiles_x, tiles_y, n_tile, n_tseg;
@@ -587,9 +587,9 @@ __global__ void __launch_bounds__(CC, 3)
 // a range of 128-channel chunks.  Per chunk the two anchors' tiles arrive by TMA ([8 x 8 tokens]
 // [channels], 128-byte swizzle) and one UMMA chain each transforms them: D[channel][column] =
 // X^T F with the tile's DFT as a 112-column operand in shared memory, M = 128 channels, K = 64
-// tokens, D in TMEM.  A thread then owns one channel: it reads both spectra from TMEM and adds
-// its products to 98 registers (Re Z, Im Z, W of 30 complex bins, Z and W of 4 real ones), which
-// are reduced over the channels once per unit.
+// tokens, D in TMEM.  A thread then owns one channel and a quarter of the bins (26 of the 98 sums: Re Z,
+// Im Z, W of 30 complex bins, Z and W of 4 real ones): it reads its columns of both spectra from TMEM
+// and adds its products in registers, which are reduced over the channels once per unit.
 // The 8x8 transform is exact: every twiddle is an integer plus an integer times sqrt(1/2), so the
 // columns hold the two integer parts (0, +-1) of each value and the thread forms A + sqrt(1/2) B
 // in f32.  Other tile shapes hold the twiddles in three bf16 pieces (24 bits), accumulated into
@@ -1536,22 +1536,22 @@ bool make_tile_map_sw(CUtensorMap* m, const cast_par_args& a, int bh) {
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// 4-D map [F][Hg][Wg][C], box (cc channels, tw, th, 1), zero fill out of range
+// f32 4-D map [F][Hg][Wg][C], box (cc channels, tw, th, 1), zero fill out of range
 bool make_r_map(CUtensorMap* m, const cast_par_args& a, int cc) {
   EncodeTiledFn fn = tensor_map_encoder();
   if (!fn) return false;
-  const cuuint64_t elt = a.dtype == CAST_BF16 ? 2 : 4;
+  const cuuint64_t elt = 4;
   cuuint64_t dims[4] = {(cuuint64_t)a.C, (cuuint64_t)a.Wg, (cuuint64_t)a.Hg, (cuuint64_t)a.F};
   cuuint64_t strides[3] = {a.C * elt, (cuuint64_t)a.Wg * a.C * elt, (cuuint64_t)a.Hg * a.Wg * a.C * elt};
   cuuint32_t box[4] = {(cuuint32_t)cc, (cuuint32_t)a.params.tile_w, (cuuint32_t)a.params.tile_h, 1};
   cuuint32_t es[4] = {1, 1, 1, 1};
-  return fn(m, a.dtype == CAST_BF16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32,
-            4, a.r, dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+  return fn(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, a.r, dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 // bf16: two launches over every tile, each a programmatic dependent of the launch before it on the
-// stream (the statistics kernel sets itself up and builds its operand while that one ends).
+// stream (behind one of this library's, the statistics kernel sets itself up and builds its operand
+// while that one ends).
 cast_status launch_tc(const CUtensorMap& tm_box, const CUtensorMap& tm_row, const CUtensorMap& tm_out, ParKArgs& k,
                       cudaStream_t st) {
   static std::atomic<uint64_t> attr_done{0};
@@ -1783,9 +1783,9 @@ ParPlan par_plan(const cast_par_args& a) {
   };
   p.n_tseg_full = segs(p.n_full, 2);
   p.n_tseg_edge = segs(p.n_edge, 4);
-  // workspace: the chunk records [tile][pair][chunk][kRec] and theta, g [tile][pair][2][kNB]
+  // workspace: the chunk records [tile][pair][chunk][kRec] and, f32, theta and g [tile][pair][2][kNB]
   p.rec_bytes = align_up((size_t)p.n_tile * (na > 0 ? na : 1) * p.n_chunk * kRec * sizeof(float));
-  p.trans_bytes = align_up((size_t)p.n_tile * (na > 0 ? na : 1) * 2 * kNB * sizeof(float));
+  p.trans_bytes = a.dtype == CAST_F32 ? align_up((size_t)p.n_tile * (na > 0 ? na : 1) * 2 * kNB * sizeof(float)) : 0;
   p.total_bytes = p.n_target > 0 ? p.rec_bytes + p.trans_bytes : 0;
   return p;
 }
@@ -1893,7 +1893,7 @@ cast_status launch_par(const cast_par_args& a, void* ws, cudaStream_t st, bool a
     // and what does not overlap with the neighbours' work, and the first one `start` more (all in
     // chunks): the statistics' reduction takes about one chunk (1,100 cycles) and their start four
     // (6,000 cycles until the first products: the DFT operand); a unit of the blend takes at least
-    // six (transport and matrices of the next one, 8,000 cycles) and the first one eight.
+    // six (transport and matrices of the next one, 6,000 to 8,000 cycles) and the first one eight.
     const int nsm = sm_count();
     auto split = [&](int64_t units, int extra, int least, int start, int& parts, int& cpp) {
       int64_t best = -1;

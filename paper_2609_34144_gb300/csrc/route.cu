@@ -1067,6 +1067,7 @@ __host__ __device__ inline WideLayout wide_layout(int na, int M, int d, int mr, 
   L.sq = refine ? take_smem(o, naf * M) : 0;
   L.G = take_smem(o, (size_t)M * sizeof(float));
   L.red2 = take_smem(o, 64 * sizeof(float));
+  // (one histogram is in use; the sizes that the entry points accept count two)
   L.hist = take_smem(o, (size_t)2 * kRadixBins * sizeof(unsigned));
   L.pre = take_smem(o, 4 * sizeof(unsigned long long));
   L.cm = restricted ? take_smem(o, (size_t)na * M) : 0;
