@@ -12,7 +12,7 @@
 //         R_t = h_a (*) R_a + h_b (*) R_b,  h = IDFT2 of the Hermitian-extended phasors
 //         phi_a = (1-alpha) e^{i g alpha theta}, phi_b = alpha e^{-i g (1-alpha) theta},
 //       so one UMMA chain per pair of targets computes [H_t1 ; H_t2] [X_a ; X_b] for 128 channels.
-//   Measured (GB300, 16 frames of 44x80 x 3072, 5 anchors): 160 -> 109 us against three launches
+//   Measured (GB300, 16 frames of 44x80 x 3072, 5 anchors): 160 -> 107 us against three launches
 //   per tile kind (register transforms, a transport that wrote the matrices, a blend that loaded
 //   them for every tile and chunk; edge tiles on a second stream).
 //
@@ -1090,12 +1090,11 @@ __global__ void __launch_bounds__(128) k_par_transport(const __grid_constant__ P
 // past, [H_t1 ; H_t2] [X_a ; X_b] per chunk (2 pieces x 8 K-steps, N = 128):
 //   warp 0       X_a and X_b of each chunk (TMA, [8 x 8 tokens][channels], the MN-major operand),
 //                four stages of 32 KB
-//   warp 2       the transport of each unit (records -> theta, g), one unit ahead
+//   warps 2, 3   the transport of each unit (records -> theta, g), alternate units, up to two ahead
 //   warps 12..15 the matrices: the convolution kernels h of the unit's targets, a table of their
 //                128 distinct 16-byte rows each, and from it one operand row per thread into TMEM
 //                (two pieces of 64 columns, two units' worth), one unit ahead of the UMMAs
-//   warps 1, 3   UMMA issuers (converged), alternate chunks, A from TMEM, D in one of two 128-column
-//                TMEM buffers
+//   warp 1       UMMA issuer (converged), A from TMEM, D in one of two 128-column TMEM buffers
 //   warps 4..11  epilogue: two sets of four warps take alternate chunks; a warp converts 32 output
 //                tokens x 64 channels at a time into one of its two 4 KB staging tiles, which it
 //                stores with TMA by itself (no barrier between warps).
@@ -1103,7 +1102,10 @@ __global__ void __launch_bounds__(128) k_par_transport(const __grid_constant__ P
 // the transport, which wrote 32 KB of matrices per (tile, target), and a blend that loaded them
 // for every (tile, chunk) - 64 KB per 32 KB of output through the ~50 bytes per clock that an SM
 // takes from L2, one staging tile for all warps - took 11 and 68 us for the full tiles of the
-// HY-World-shaped call, 9.5 and 19 us beside them for the edge tiles.  With the matrices in shared
+// HY-World-shaped call, 9.5 and 19 us beside them for the edge tiles.  A unit's transport is one chain
+// of ~5,500 cycles, its matrices take ~3,500: with one transport warp (and a second issuer in place of
+// the other) a unit could not take less than six chunks (HY-World-shaped call 109 -> 107 us, with 4x4
+// tiles 388 -> 339 us).  With the matrices in shared
 // memory the UMMAs read both operands from there (128 bytes per clock, as much as an SM has).
 constexpr int kTbStages = 4;
 constexpr int kTbPlane = 64 * 128 * 2;          // one anchor tile of a chunk, 16 KB
@@ -1192,8 +1194,8 @@ __global__ void __launch_bounds__(kTbThreads, 1)
   uint8_t* s_out = dsm + kTbStages * kTbStage;
   MatrixShared& m = *reinterpret_cast<MatrixShared*>(s_out + 16 * kTbOut);
   __shared__ __align__(8) uint64_t b_xfull[kTbStages], b_xempty[kTbStages], b_mfull[2], b_mempty[2], b_dfull[2],
-      b_dempty[2], b_tready, b_tfree;
-  __shared__ float s_th[kNB], s_gate[kNB];   // of the unit whose matrices are next
+      b_dempty[2], b_tready[2], b_tfree[2];
+  __shared__ float s_th[2][kNB], s_gate[2][kNB];   // of the units whose matrices are next
   __shared__ uint32_t s_tmem;
   __shared__ volatile int s_abort;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -1213,12 +1215,12 @@ __global__ void __launch_bounds__(kTbThreads, 1)
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(&b_mfull[b], 128);
-      mbar_init(&b_mempty[b], 2);   // both issuers
+      mbar_init(&b_mempty[b], 1);
+      mbar_init(&b_tready[b], 1);
+      mbar_init(&b_tfree[b], 1);
       mbar_init(&b_dfull[b], 1);
       mbar_init(&b_dempty[b], 4);
     }
-    mbar_init(&b_tready, 1);
-    mbar_init(&b_tfree, 1);
     fence_barrier_init();
     s_abort = 0;
   }
@@ -1231,7 +1233,7 @@ __global__ void __launch_bounds__(kTbThreads, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = s_tmem;
-  // (the warps that read what earlier launches wrote, 0 and 2, wait for the grid before)
+  // (the warps that read what earlier launches wrote, 0, 2 and 3, wait for the grid before)
   const int n_part = a.bl_parts, n_item = a.n_grp;   // an item: up to two targets of a pair
   const auto c0_of = [&](const Unit& u) { return u.part * a.bl_cpp; };
   const auto c1_of = [&](const Unit& u) { return min(a.n_chunk, (u.part + 1) * a.bl_cpp); };
@@ -1286,7 +1288,7 @@ __global__ void __launch_bounds__(kTbThreads, 1)
         }
       }
       // (the four warps leave together)
-      if (bar_sync_or(3, 128, !wait(&b_tready, (uint32_t)k & 1u))) break;
+      if (bar_sync_or(3, 128, !wait(&b_tready[k & 1], (uint32_t)(k >> 1) & 1u))) break;
       if (mt < 2 * kNB) {
         const int ts = mt / kNB, b = mt - ts * kNB, ky = b / 5, kx = b % 5;
         float4 ph = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -1295,7 +1297,7 @@ __global__ void __launch_bounds__(kTbThreads, 1)
           const bool edge = kx == 0 || ((w % 2 == 0) && kx == w / 2);
           const float kap = (edge ? 1.f : 2.f) / (float)(h * w);
           float sa, ca, sb, cb;
-          const float gt = s_gate[b] * s_th[b];
+          const float gt = s_gate[k & 1][b] * s_th[k & 1][b];
           sincosf(gt * al, &sa, &ca);
           sincosf(-gt * (1.f - al), &sb, &cb);
           ph = make_float4(kap * (1.f - al) * ca, kap * (1.f - al) * sa, kap * al * cb, kap * al * sb);
@@ -1303,7 +1305,7 @@ __global__ void __launch_bounds__(kTbThreads, 1)
         m.phi[ts][b] = ph;
       }
       matrix_sync();
-      if (mt == 0) mbar_arrive(&b_tfree);   // theta and g have been read
+      if (mt == 0) mbar_arrive(&b_tfree[k & 1]);   // theta and g have been read
 #pragma unroll
       for (int ts = 0; ts < 2; ++ts) {
         float cr = 0.f, ci = 0.f;
@@ -1373,35 +1375,36 @@ __global__ void __launch_bounds__(kTbThreads, 1)
       tc_fence_before();
       mbar_arrive(&b_mfull[mb]);
     }
-  } else if (warp == 2) {
+  } else if (warp == 2 || warp == 3) {
     // ---------------------------------------------------------------- transport
-    __shared__ TransportShared ms;
+    // warps 2 and 3 take alternate units
+    __shared__ TransportShared both[2];
+    const int me = warp & 1;
+    TransportShared& ms = both[me];
     int k = 0, shape = -1, at[kZwPer];
     for (Unit x = first_unit(n_part, n_item); x.tile < a.n_tile; next_unit(x, a.bl_step, n_part, n_item), ++k) {
+      if ((k & 1) != me) continue;
       const TileGeom g = any_tile(a, x.tile);
       const bool fresh = g.h * 16 + g.w != shape;
       shape = g.h * 16 + g.w;
       if (fresh) transport_shape(a, g, ms, at, lane);
-      if (k == 0) grid_dependency_wait();   // the records of K_stats_tc
-      // only the hand-over waits for the matrix warps to have read the unit before (the transport
-      // takes ~5,000 cycles, their reading of it ~2,000)
+      if (k == me) grid_dependency_wait();   // the records of K_stats_tc
       float th[2], gate[2];
       unit_transport(a, g, x.tile, a.grp_pair[x.item], ms, at, th, gate, lane);
-      if (!__all_sync(0xffffffffu, k == 0 || wait(&b_tfree, (uint32_t)(k - 1) & 1u))) break;
+      // only the hand-over waits for the matrix warps to have read the unit before the last
+      if (!__all_sync(0xffffffffu, k < 2 || wait(&b_tfree[me], (uint32_t)((k >> 1) - 1) & 1u))) break;
 #pragma unroll
       for (int s = 0; s < 2; ++s)
         if (lane + 32 * s < kNB) {
-          s_th[lane + 32 * s] = th[s];
-          s_gate[lane + 32 * s] = gate[s];
+          s_th[me][lane + 32 * s] = th[s];
+          s_gate[me][lane + 32 * s] = gate[s];
         }
       __syncwarp();
-      if (lane == 0) mbar_arrive(&b_tready);
+      if (lane == 0) mbar_arrive(&b_tready[me]);
     }
   } else if (warp < 4) {
-    // ---------------------------------------------------------------- UMMA issuers (converged)
-    // warps 1 and 3 take alternate chunks and accumulators (see K_stats_tc)
+    // ---------------------------------------------------------------- UMMA issuer (converged)
     constexpr uint32_t idesc = idesc_bf16_f32(128, 128, false, true);
-    const int buf = warp >> 1;
     const uint32_t tmu = __shfl_sync(0xffffffffu, tmem, 0);
     const uint32_t xb = __shfl_sync(0xffffffffu, smem_u32(s_x), 0);
     const uint64_t dx = sdesc_sw128(xb, 8192, 1024);
@@ -1413,8 +1416,7 @@ __global__ void __launch_bounds__(kTbThreads, 1)
       if (!(ok = __all_sync(0xffffffffu, wait(&b_mfull[mb], (uint32_t)(k >> 1) & 1u)))) break;
       tc_fence_after();
       for (int c = c0_of(x), c1 = c1_of(x); c < c1; ++c, ++n) {
-        if ((n & 1) != buf) continue;
-        const int s = n % kTbStages;
+        const int s = n % kTbStages, buf = n & 1;
         // half of the warp waits for the anchors, half for the accumulator
         const bool w = lane < 16 ? wait(&b_xfull[s], (uint32_t)(n / kTbStages) & 1u)
                                  : n < 2 || wait(&b_dempty[buf], (uint32_t)((n >> 1) - 1) & 1u);
@@ -1435,12 +1437,12 @@ __global__ void __launch_bounds__(kTbThreads, 1)
         __syncwarp();
         last = n;
       }
-      // this issuer's last reads of the unit's matrices
+      // the last reads of the unit's matrices
       if (ok && lead) umma_commit(&b_mempty[mb]);
       __syncwarp();
     }
     // the UMMAs issued so far have completed before shared memory and TMEM are released
-    if (last >= 0) mbar_wait(&b_dfull[buf], (uint32_t)(last >> 1) & 1u, lim);
+    if (last >= 0) mbar_wait(&b_dfull[last & 1], (uint32_t)(last >> 1) & 1u, lim);
     __syncwarp();
   } else if (warp >= 4) {   // 4..11
     // ---------------------------------------------------------------- epilogue
@@ -1892,8 +1894,9 @@ cast_status launch_par(const cast_par_args& a, void* ws, cudaStream_t st, bool a
     // lose the anchors' reuse in L2: HY-World-shaped 109 -> 123 us); a unit takes its chunks
     // and what does not overlap with the neighbours' work, and the first one `start` more (all in
     // chunks): the statistics' reduction takes about one chunk (1,100 cycles) and their start four
-    // (6,000 cycles until the first products: the DFT operand); a unit of the blend takes at least
-    // six (transport and matrices of the next one, 6,000 to 8,000 cycles) and the first one eight.
+    // (6,000 cycles until the first products: the DFT operand); a unit of the blend counts as at least
+    // six (3, 4 or 5 give the HY-World-shaped call 124 / 107 / 108 us and one with 8 anchors 141 / 142 /
+    // 140, six 107 and 132) and the first one eight.
     const int nsm = sm_count();
     auto split = [&](int64_t units, int extra, int least, int start, int& parts, int& cpp) {
       int64_t best = -1;
