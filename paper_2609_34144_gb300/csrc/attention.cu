@@ -309,13 +309,14 @@ __global__ void __launch_bounds__(kThreads, 1)
           tma_load_3d(sQ + t * C::Q_BYTES + b * BM * 128, &tm_q, &bars->q_full, h * HD + b * 64,
                       row0 + t * BM, a.q_frame[i]);
       bool waited = false;
-      int j = 0;
-      for (; j < n_tiles; ++j) {
+      int loads = n_tiles;
+      for (int j = 0; j < n_tiles; ++j) {
         if (k0 + j >= a.n_cur_tiles) wait_routing(waited);
         const TileCoord c = tile_coord(a, i, h, k0 + j);
         const int s = j % kStages;
         if (aborted(bars) || !mbar_wait(&bars->k_empty[s], ((uint32_t)(j / kStages) & 1u) ^ 1u, lim)) {
           set_abort(bars);
+          loads = j;
           break;
         }
         mbar_arrive_expect_tx(&bars->k_full[s], C::KV_BYTES);
@@ -338,20 +339,21 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
       // (also after a timeout) what was loaded last has landed before shared memory is released
       mbar_wait(&bars->q_full, 0, lim);
-      for (int l = max(0, j - kStages); l < j; ++l) mbar_wait(&bars->k_full[l % kStages], (uint32_t)(l / kStages) & 1u, lim);
+      for (int l = max(0, loads - kStages); l < loads; ++l) mbar_wait(&bars->k_full[l % kStages], (uint32_t)(l / kStages) & 1u, lim);
     }
   } else if (warp == 2) {
     if (lane == 0) {
       tma_prefetch_desc(&tm_vc);
       tma_prefetch_desc(&tm_vh);
       bool waited = false;
-      int j = 0;
-      for (; j < n_tiles; ++j) {
+      int loads = n_tiles;
+      for (int j = 0; j < n_tiles; ++j) {
         if (k0 + j >= a.n_cur_tiles) wait_routing(waited);
         const TileCoord c = tile_coord(a, i, h, k0 + j);
         const int s = j % kStages;
         if (aborted(bars) || !mbar_wait(&bars->v_empty[s], ((uint32_t)(j / kStages) & 1u) ^ 1u, lim)) {
           set_abort(bars);
+          loads = j;
           break;
         }
         mbar_arrive_expect_tx(&bars->v_full[s], C::KV_BYTES);
@@ -372,7 +374,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           }
         }
       }
-      for (int l = max(0, j - kStages); l < j; ++l) mbar_wait(&bars->v_full[l % kStages], (uint32_t)(l / kStages) & 1u, lim);
+      for (int l = max(0, loads - kStages); l < loads; ++l) mbar_wait(&bars->v_full[l % kStages], (uint32_t)(l / kStages) & 1u, lim);
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ UMMA issuer
