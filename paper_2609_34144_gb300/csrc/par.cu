@@ -1684,6 +1684,7 @@ class ForkLease {
     } else {
       if (f_.fork) cudaEventDestroy(f_.fork);
       if (f_.side) cudaStreamDestroy(f_.side);
+      cudaGetLastError();   // (the call goes on without a side stream)
     }
     cudaThreadExchangeStreamCaptureMode(&mode);
   }
